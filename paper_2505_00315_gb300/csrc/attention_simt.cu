@@ -120,7 +120,7 @@ attn_bwd_dq_simt_kernel(const void *__restrict__ Q, const void *__restrict__ K,
     }
     if (i < k) {
 #pragma unroll
-        for (int p = 0; p < HP; ++p) Inter<TS>::st(dQKV, base + i, 3 * HP, p, dq[p] * scale);
+        for (int p = 0; p < HP; ++p) Inter<TS>::st(dQKV, base + i, 4 * HP, p, dq[p] * scale);
     }
 }
 
@@ -179,7 +179,7 @@ attn_bwd_dkv_simt_kernel(const void *__restrict__ Q, const void *__restrict__ K,
         const int col = kDK ? HP : 2 * HP;
         const float f = kDK ? scale : 1.f;
 #pragma unroll
-        for (int p = 0; p < HP; ++p) Inter<TS>::st(dQKV, base + j, 3 * HP, col + p, acc[p] * f);
+        for (int p = 0; p < HP; ++p) Inter<TS>::st(dQKV, base + j, 4 * HP, col + p, acc[p] * f);
     }
 }
 

@@ -65,7 +65,7 @@ size_t carve(const Dims &dm, char *base, Saved *sv) {
     s.dA = take(e * R * dm.hp);
     s.dlogit = (float *)take(sizeof(float) * R);
     s.Dd = (float *)take(sizeof(float) * R);
-    s.dQKV = take(e * R * 4 * dm.hp);  // 3 h' columns, or 4 blocks of 64 on the tensor cores
+    s.dQKV = take(e * R * 4 * dm.hp);  // dQ | dK | dV | dlogit
     s.G = (float *)take(sizeof(float) * R * dm.hp);
     s.WrT = (float *)take(sizeof(float) * (size_t)dm.d * dm.H);
     // (reserved for either dtype, so that the size depends on the shape only)
@@ -150,16 +150,14 @@ cudaError_t link(cudaStream_t from, cudaStream_t to, cudaEvent_t ev) {
 // F3-F5 for the rows already selected into sv.gidx / sv.rsel.
 // RoPE (Sec. 2.2) in place on the stored Q and K rows (dir +1), or on the dQ
 // and dK blocks of the dQ|dK|dV rows (dir -1).  Pair storage for bf16 inputs:
-// on the tensor cores Q is [hi 64 | lo 64] and dQ|dK|dV|dlogit [hi 256 | lo 256]
-// per row, on the CUDA cores [hi hp | lo hp] and [hi 3hp | lo 3hp]; fp32 rows
-// otherwise.
+// Q is [hi hp | lo hp] and dQ|dK|dV|dlogit [hi 4hp | lo 4hp] per row; fp32
+// rows otherwise.
 cudaError_t rope_qk(const Dims &dm, const Saved &sv, bool grads, cudaStream_t s) {
     const RopeTable tab = make_rope_table(dm.hp, dm.T);
     const long long rows = dm.rows();
     const bool pair = dm.bf16;
     if (!grads) return launch_rope(sv.Q, 0, sv.K, 0, pair, dm.hp, rows, sv.gidx, tab, 1.f, s);
-    const int cols = use_tc(dm) ? 256 : 3 * dm.hp;
-    return launch_rope(sv.dQKV, 0, sv.dQKV, dm.hp, pair, cols, rows, sv.gidx, tab, -1.f, s);
+    return launch_rope(sv.dQKV, 0, sv.dQKV, dm.hp, pair, 4 * dm.hp, rows, sv.gidx, tab, -1.f, s);
 }
 
 mosa_status forward_heads(const Dims &dm, const void *X, const void *W_q, const void *W_k,
@@ -544,7 +542,7 @@ bool graphs_enabled() {
 
 int path_bits(const Dims &dm) {
     return (use_tc(dm) ? 1 : 0) | (use_fused_forward(dm) ? 2 : 0) | (use_fused_backward(dm) ? 4 : 0) |
-           (use_headsum_out(dm) ? 8 : 0) | (use_headsum_dx(dm) ? 16 : 0);
+           (use_headsum_out(dm) ? 8 : 0) | (use_headsum_dx(dm) ? 16 : 0) | (use_split() ? 32 : 0);
 }
 
 GraphKey make_key(int op, const Dims &dm, const mosa_shape *shape,
@@ -554,7 +552,7 @@ GraphKey make_key(int op, const Dims &dm, const mosa_shape *shape,
     std::memset(&k, 0, sizeof(k));
     k.op = op;
     cudaGetDevice(&k.device);
-    k.tc = path_bits(dm) | (dense ? path_bits(*dense) << 5 : 0);
+    k.tc = path_bits(dm) | (dense ? path_bits(*dense) << 6 : 0);
     k.mask = profile_mask();
     k.shape = *shape;
     k.extra[0] = extra0;
@@ -789,13 +787,13 @@ int32_t mosa_stage_engine(const mosa_shape *shape, int32_t stage) {
     if (check_shape(shape, &dm) != MOSA_OK || stage < 0 || stage >= kNumStages) return -1;
     switch (stage) {
         case kStageRouter: return (use_tc(dm) && dm.H % 8 == 0) ? 1 : 0;
-        case kStageSelect: return 2;
         case kStageQkv:
         case kStageOut:
         case kStageOutBwd:
         case kStageInBwd:
         case kStageWBwd:
-        case kStageDwo:
+        case kStageDwo: return use_split() ? 1 : 0;
+        case kStageSelect: return 2;
         case kStageAttnFwd:
         case kStageAttnBwd: return use_tc(dm) ? 1 : 0;
         case kStageFwdUnit: return use_fused_forward(dm) ? 1 : 0;

@@ -1,141 +1,261 @@
-// Per-head projections of the MoSA layer on CUDA cores (fp32 FFMA), used for
-// fp32 storage and as the plain path for bf16:
+// Per-head projections of the MoSA layer for fp32 storage and for bf16 with a
+// head size other than 64 (and, with MOSA_FORCE_SIMT, for every shape):
 //   F3  Q, K, V = X^s W^{Q,K,V}           (X^s = X[b, I, :], Sec. 2.2)
 //   F5  Y[b, I, :] += diag(r^topk) A W^o  (scatter-sum over heads, Eq. mosa_mha)
 //   B1  G = dY[I] W^o^T, dW^o = (diag(r) A)^T dY[I], and the row terms
 //       dr = <A, G>, dA = r G, dlogit = dr r (1 - r), D = rowsum(dA o A)
 //   B3  dX[b, I, :] += dQ W^Q^T + dK W^K^T + dV W^V^T + dlogit W^r[:,h]^T
 //   B4  dW^{Q,K,V} = X^s^T d{Q,K,V},  dW^r[:,h] = X^s^T dlogit
-// Rows of head h are m = b*k + i; gidx maps them to rows of X / Y / dY.
+// Rows of head h are m = b*k + i; gidx maps them to rows of X / Y / dY.  Each
+// product is described once (an Op) and runs on the tensor cores through bf16
+// planes (tc_split.cuh), or on the CUDA cores (simt_gemm.cuh) when forced or
+// when a tensor's address is not 16-byte aligned.
+// dQ|dK|dV rows have 4 h' columns: 3 h' of gradients, then dlogit (bf16: its
+// pair at column 3 h' and the pair of what that rounded off at 3 h' + 1).
 #include <cstdlib>
+#include <initializer_list>
+#include <type_traits>
 
 #include "launch.h"
 #include "simt_gemm.cuh"
+#include "tc_split.cuh"
 
 namespace mosa {
 namespace {
 
+// Planes of an input tensor and of a stored intermediate of storage type T.
+template <class T>
+constexpr int in_planes() { return sizeof(T) == 4 ? 3 : 1; }
+template <class T>
+constexpr int inter_planes() { return sizeof(T) == 4 ? 3 : 2; }
+// Elements per stored intermediate row of `cols` columns.
+template <class T>
+constexpr int inter_ld(int cols) { return sizeof(T) == 4 ? cols : 2 * cols; }
+
+// Four consecutive columns of an intermediate row (Inter<TS>::st of each).
+template <class T>
+__device__ __forceinline__ void st_inter4(void *p, size_t row, int cols, int c, const float4 &v) {
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4 *>(static_cast<float *>(p) + row * cols + c) = v;
+    } else {
+        const float x[4] = {v.x, v.y, v.z, v.w};
+        __nv_bfloat162 hi[2], lo[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const bf16 h0 = __float2bfloat16_rn(x[2 * e]), h1 = __float2bfloat16_rn(x[2 * e + 1]);
+            hi[e] = __halves2bfloat162(h0, h1);
+            lo[e] = __halves2bfloat162(__float2bfloat16_rn(x[2 * e] - __bfloat162float(h0)),
+                                       __float2bfloat16_rn(x[2 * e + 1] - __bfloat162float(h1)));
+        }
+        bf16 *q = static_cast<bf16 *>(p) + row * 2 * cols + c;
+        *reinterpret_cast<uint2 *>(q) = *reinterpret_cast<const uint2 *>(hi);
+        *reinterpret_cast<uint2 *>(q + cols) = *reinterpret_cast<const uint2 *>(lo);
+    }
+}
+
+// The result of one reduction split: four columns, or one value.
+__device__ __forceinline__ void put4(float *dst, const float4 &v, bool add) {
+    if (add)
+        tc::red_add_v4(dst, v.x, v.y, v.z, v.w);
+    else
+        *reinterpret_cast<float4 *>(dst) = v;
+}
+__device__ __forceinline__ void put1(float *dst, float v, bool add) {
+    if (add)
+        atomicAdd(dst, v);
+    else
+        *dst = v;
+}
+
 template <class T>
 struct QkvOp {
     using TS = typename InterOf<T>::type;
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = true, kBKFast = false;
+    static constexpr int kPA = in_planes<T>(), kPB = in_planes<T>();
+    static constexpr bool kAMN = false, kBMN = true, kTrans = false;
     int M, N, K;  // B*k, 3*hp, d
-    int hp;
-    const T *X, *Wq, *Wk, *Wv;
+    int hp, lg;   // lg: log2 hp
+    const T *A;   // X
+    const T *Wq, *Wk, *Wv;
     const int32_t *gidx;
     void *Q, *Kp, *V;
-    __device__ float a(int g, int m, int c) const {
-        return to_f32(X[(size_t)gidx[(size_t)g * M + m] * K + c]);
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return gidx[(size_t)g * M + m]; }
+    __device__ const T *b_ptr(int g, int c, int n) const {
+        const int w = n >> lg, p = n & (hp - 1);
+        return (w == 0 ? Wq : (w == 1 ? Wk : Wv)) + ((size_t)g * K + c) * hp + p;
     }
-    __device__ float b(int g, int c, int n) const {
-        const int w = n / hp, p = n - w * hp;
-        const T *W = w == 0 ? Wq : (w == 1 ? Wk : Wv);
-        return to_f32(W[((size_t)g * K + c) * hp + p]);
+    __device__ float a(int g, int m, int c) const { return to_f32(A[(size_t)a_row(g, m) * K + c]); }
+    __device__ float b(int g, int c, int n) const { return to_f32(*b_ptr(g, c, n)); }
+    __device__ void store(int g, int m, int n, float v, bool) const {
+        const int w = n >> lg, p = n & (hp - 1);
+        Inter<TS>::st(w == 0 ? Q : (w == 1 ? Kp : V), (size_t)g * M + m, hp, p, v);
     }
-    __device__ void store(int g, int m, int n, float v) const {
-        const int w = n / hp, p = n - w * hp;
-        void *O = w == 0 ? Q : (w == 1 ? Kp : V);
-        Inter<TS>::st(O, (size_t)g * M + m, hp, p, v);
+    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+        const int w = n >> lg, p = n & (hp - 1);
+        st_inter4<T>(w == 0 ? Q : (w == 1 ? Kp : V), (size_t)g * M + m, hp, p, v);
     }
 };
 
 template <class T>
 struct OutOp {
     using TS = typename InterOf<T>::type;
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = true, kBKFast = false;
+    static constexpr int kPA = inter_planes<T>(), kPB = in_planes<T>();
+    static constexpr bool kAMN = false, kBMN = true, kTrans = false;
     int M, N, K;  // B*k, d, hp
-    const void *AR;
+    const T *A;   // AR rows
     const T *Wo;
     const int32_t *gidx;
     float *Y;
-    __device__ float a(int g, int m, int p) const { return Inter<TS>::ld(AR, (size_t)g * M + m, K, p); }
-    __device__ float b(int g, int p, int n) const { return to_f32(Wo[((size_t)g * K + p) * N + n]); }
-    __device__ void store(int g, int m, int n, float v) const {
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return g * M + m; }
+    __device__ const T *b_ptr(int g, int p, int n) const { return Wo + ((size_t)g * K + p) * N + n; }
+    __device__ float a(int g, int m, int p) const { return Inter<TS>::ld(A, (size_t)g * M + m, K, p); }
+    __device__ float b(int g, int p, int n) const { return to_f32(*b_ptr(g, p, n)); }
+    __device__ void store(int g, int m, int n, float v, bool) const {
         atomicAdd(Y + (size_t)gidx[(size_t)g * M + m] * N + n, v);
+    }
+    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+        tc::red_add_v4(Y + (size_t)gidx[(size_t)g * M + m] * N + n, v.x, v.y, v.z, v.w);
     }
 };
 
 template <class T>
 struct OutBwdGOp {
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = true, kBKFast = true;
+    static constexpr int kPA = in_planes<T>(), kPB = in_planes<T>();
+    static constexpr bool kAMN = false, kBMN = false, kTrans = false;
     int M, N, K;  // B*k, hp, d
-    const T *dY, *Wo;
+    const T *A;   // dY
+    const T *Wo;
     const int32_t *gidx;
     float *G;
-    __device__ float a(int g, int m, int c) const {
-        return to_f32(dY[(size_t)gidx[(size_t)g * M + m] * K + c]);
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return gidx[(size_t)g * M + m]; }
+    __device__ const T *b_ptr(int g, int n, int c) const { return Wo + ((size_t)g * N + n) * K + c; }
+    __device__ float a(int g, int m, int c) const { return to_f32(A[(size_t)a_row(g, m) * K + c]); }
+    __device__ float b(int g, int c, int n) const { return to_f32(*b_ptr(g, n, c)); }
+    __device__ void store(int g, int m, int n, float v, bool) const { G[((size_t)g * M + m) * N + n] = v; }
+    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+        *reinterpret_cast<float4 *>(G + ((size_t)g * M + m) * N + n) = v;
     }
-    __device__ float b(int g, int c, int n) const { return to_f32(Wo[((size_t)g * N + n) * K + c]); }
-    __device__ void store(int g, int m, int n, float v) const { G[((size_t)g * M + m) * N + n] = v; }
 };
 
+// dW_o[h](p, c): rows c of d, columns p, reduced over the head's rows.
 template <class T>
 struct OutBwdWOp {
     using TS = typename InterOf<T>::type;
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = false, kBKFast = false;
-    int M, N, K;  // hp, d, B*k
-    const void *AR;
-    const T *dY;
+    static constexpr int kPA = in_planes<T>(), kPB = inter_planes<T>();
+    static constexpr bool kAMN = true, kBMN = true, kTrans = true;
+    int M, N, K;  // d, hp, B*k
+    const T *A;   // dY
+    const T *AR;
     const int32_t *gidx;
     float *dWo;
-    __device__ float a(int g, int p, int m) const { return Inter<TS>::ld(AR, (size_t)g * K + m, M, p); }
-    __device__ float b(int g, int m, int n) const {
-        return to_f32(dY[(size_t)gidx[(size_t)g * K + m] * N + n]);
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return gidx[(size_t)g * K + m]; }
+    __device__ const T *b_ptr(int g, int m, int p) const {
+        return AR + ((size_t)g * K + m) * inter_ld<T>(N) + p;
     }
-    __device__ void store(int g, int p, int n, float v) const { dWo[((size_t)g * M + p) * N + n] = v; }
+    __device__ float a(int g, int c, int m) const { return to_f32(A[(size_t)a_row(g, m) * M + c]); }
+    __device__ float b(int g, int m, int p) const { return Inter<TS>::ld(AR, (size_t)g * K + m, N, p); }
+    __device__ void store(int g, int c, int p, float v, bool add) const {
+        put1(dWo + ((size_t)g * N + p) * M + c, v, add);
+    }
+    __device__ void store4(int, int, int, const float4 &, bool) const {}
 };
 
 template <class T>
 struct InBwdOp {
     using TS = typename InterOf<T>::type;
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = true, kBKFast = true;
+    static constexpr int kPA = inter_planes<T>(), kPB = in_planes<T>();
+    static constexpr bool kAMN = false, kBMN = false, kTrans = false;
     int M, N, K;  // B*k, d, 3*hp
-    int hp, H;
-    const void *dQKV;
+    int hp, lg, H;   // lg: log2 hp
+    const T *A;   // dQ|dK|dV rows
     const T *Wq, *Wk, *Wv, *Wr;
     const float *dlogit;
     const int32_t *gidx;
     float *dX;
-    __device__ float a(int g, int m, int kk) const { return Inter<TS>::ld(dQKV, (size_t)g * M + m, K, kk); }
-    __device__ float b(int g, int kk, int n) const {
-        const int w = kk / hp, p = kk - w * hp;
-        const T *W = w == 0 ? Wq : (w == 1 ? Wk : Wv);
-        return to_f32(W[((size_t)g * N + n) * hp + p]);
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return g * M + m; }
+    __device__ const T *b_ptr(int g, int n, int kk) const {
+        const int w = kk >> lg, p = kk & (hp - 1);
+        return (w == 0 ? Wq : (w == 1 ? Wk : Wv)) + ((size_t)g * N + n) * hp + p;
     }
-    __device__ void store(int g, int m, int n, float v) const {
+    __device__ float a(int g, int m, int kk) const { return Inter<TS>::ld(A, (size_t)g * M + m, 4 * hp, kk); }
+    __device__ float b(int g, int kk, int n) const { return to_f32(*b_ptr(g, n, kk)); }
+    __device__ void store(int g, int m, int n, float v, bool) const {
         const size_t row = (size_t)g * M + m;
         v = fmaf(dlogit[row], to_f32(Wr[(size_t)n * H + g]), v);
         atomicAdd(dX + (size_t)gidx[row] * N + n, v);
     }
+    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+        const size_t row = (size_t)g * M + m;
+        const float dl = dlogit[row];
+        const T *w = Wr + (size_t)n * H + g;
+        tc::red_add_v4(dX + (size_t)gidx[row] * N + n, fmaf(dl, to_f32(w[0]), v.x),
+                       fmaf(dl, to_f32(w[H]), v.y), fmaf(dl, to_f32(w[2 * (size_t)H]), v.z),
+                       fmaf(dl, to_f32(w[3 * (size_t)H]), v.w));
+    }
 };
 
-// dW_{q,k,v} and, as one extra output column, dW_r.
+// dW_{q,k,v} and, from the dlogit columns of the rows, dW_r.
 template <class T>
 struct WBwdOp {
     using TS = typename InterOf<T>::type;
+    using TA = T;
+    using TB = T;
     static constexpr bool kAKFast = false, kBKFast = false;
-    int M, N, K;  // d, 3*hp + 1, B*k
-    int hp, H;
-    const T *X;
-    const void *dQKV;
+    static constexpr int kPA = in_planes<T>(), kPB = inter_planes<T>();
+    static constexpr bool kAMN = true, kBMN = true, kTrans = false;
+    static constexpr int kExtra = sizeof(T) == 4 ? 1 : 2;   // dlogit columns
+    int M, N, K;  // d, 3*hp + kExtra, B*k
+    int hp, lg, H;   // lg: log2 hp
+    const T *A;   // X
+    const T *dQKV;
     const float *dlogit;
     const int32_t *gidx;
     float *dWq, *dWk, *dWv, *dWr;
-    __device__ float a(int g, int c, int m) const {
-        return to_f32(X[(size_t)gidx[(size_t)g * K + m] * M + c]);
+    int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
+    __device__ int a_row(int g, int m) const { return gidx[(size_t)g * K + m]; }
+    __device__ const T *b_ptr(int g, int m, int n) const {
+        return dQKV + ((size_t)g * K + m) * inter_ld<T>(4 * hp) + n;
     }
+    __device__ float a(int g, int c, int m) const { return to_f32(A[(size_t)a_row(g, m) * M + c]); }
     __device__ float b(int g, int m, int n) const {
         const size_t row = (size_t)g * K + m;
-        return n < 3 * hp ? Inter<TS>::ld(dQKV, row, 3 * hp, n) : dlogit[row];
+        if (n > 3 * hp) return 0.f;   // (dlogit's rounding remainder, in its fp32 value already)
+        return n < 3 * hp ? Inter<TS>::ld(dQKV, row, 4 * hp, n) : dlogit[row];
     }
-    __device__ void store(int g, int c, int n, float v) const {
-        if (n == 3 * hp) {
-            dWr[(size_t)c * H + g] = v;
-            return;
-        }
-        const int w = n / hp, p = n - w * hp;
-        float *O = w == 0 ? dWq : (w == 1 ? dWk : dWv);
-        O[((size_t)g * M + c) * hp + p] = v;
+    __device__ float *dst(int g, int c, int n) const {
+        const int w = n >> lg, p = n & (hp - 1);
+        return (w == 0 ? dWq : (w == 1 ? dWk : dWv)) + ((size_t)g * M + c) * hp + p;
+    }
+    __device__ void store(int g, int c, int n, float v, bool add) const {
+        if (n < 3 * hp)
+            put1(dst(g, c, n), v, add);
+        else if (n == 3 * hp)
+            put1(dWr + (size_t)c * H + g, v, add);
+    }
+    __device__ void store4(int g, int c, int n, const float4 &v, bool add) const {
+        if (n < 3 * hp)
+            put4(dst(g, c, n), v, add);
+        else
+            put1(dWr + (size_t)c * H + g, kExtra == 2 ? v.x + v.y : v.x, add);
     }
 };
 
@@ -145,7 +265,8 @@ template <class TS>
 __global__ void out_bwd_rows_kernel(const float *__restrict__ G, const float *__restrict__ A,
                                     const float *__restrict__ rsel, void *__restrict__ dA,
                                     float *__restrict__ Dd, float *__restrict__ dlogit,
-                                    long long rows, int hp) {
+                                    void *__restrict__ dQKV, long long rows, int hp) {
+    tc::pdl_wait();
     const long long row = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (row >= rows) return;
@@ -165,105 +286,142 @@ __global__ void out_bwd_rows_kernel(const float *__restrict__ G, const float *__
         dd += __shfl_xor_sync(0xffffffffu, dd, off);
     }
     if (lane == 0) {
+        const float dl = dr * r * (1.f - r);
         Dd[row] = dd;
-        dlogit[row] = dr * r * (1.f - r);
+        dlogit[row] = dl;
+        if constexpr (std::is_same<TS, float>::value) {
+            static_cast<float *>(dQKV)[row * 4 * hp + 3 * hp] = dl;
+        } else {
+            // three bf16 parts (a non-finite value only in the first)
+            bf16 *q = static_cast<bf16 *>(dQKV) + row * 8 * hp + 3 * hp;
+            const bf16 h = __float2bfloat16_rn(dl);
+            const float r1 = fabsf(dl) <= 3.38e38f ? dl - __bfloat162float(h) : 0.f;
+            const bf16 l = __float2bfloat16_rn(r1);
+            q[0] = h;
+            q[4 * hp] = l;
+            q[1] = __float2bfloat16_rn(r1 - __bfloat162float(l));
+            q[4 * hp + 1] = __float2bfloat16_rn(0.f);
+        }
     }
 }
 
-// dW_r[c, h] = sum_m X[g(m), c] dlogit(m): one thread per column c of one
-// head and one slice of the rows; slices are summed with atomics.
-template <class T>
-__global__ void dwr_kernel(const T *__restrict__ X, const int32_t *__restrict__ gidx,
-                           const float *__restrict__ dlogit, float *__restrict__ dWr, int Mtok,
-                           int d, int H, int rows_per_slice) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int h = blockIdx.y;
-    const int m_begin = blockIdx.z * rows_per_slice;
-    const int m_end = min(Mtok, m_begin + rows_per_slice);
-    if (c >= d) return;
-    float acc = 0.f;
-    for (int m = m_begin; m < m_end; ++m) {
-        const size_t row = (size_t)h * Mtok + m;
-        acc = fmaf(to_f32(X[(size_t)gidx[row] * d + c]), dlogit[row], acc);
-    }
-    atomicAdd(dWr + (size_t)c * H + h, acc);
+bool aligned16(std::initializer_list<const void *> ps) {
+    uintptr_t u = 0;
+    for (const void *p : ps) u |= reinterpret_cast<uintptr_t>(p);
+    return (u & 15) == 0;
 }
 
-template <class T>
-cudaError_t dwr_t(const Dims &dm, const void *X, const Saved &sv, float *dWr, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(dWr, 0, sizeof(float) * (size_t)dm.d * dm.H, s);
-    if (e != cudaSuccess) return e;
-    const int Mtok = dm.B * dm.k;
-    const int rows = 64;
-    dim3 grid((dm.d + 255) / 256, dm.H, (Mtok + rows - 1) / rows);
-    dwr_kernel<T><<<grid, 256, 0, s>>>((const T *)X, sv.gidx, sv.dlogit, dWr, Mtok, dm.d, dm.H,
-                                       rows);
-    note_launches(1);
-    return cudaGetLastError();
+// One product on the tensor cores (split), or on the CUDA cores.
+template <class Op>
+cudaError_t product(const Op &op, int groups, int splits, bool split, const Saved &sv,
+                    cudaStream_t s) {
+    return split ? launch_split_gemm(op, groups, splits, sv.status, s)
+                 : launch_simt_gemm(op, groups, s);
+}
+
+int log2_of(int hp) {   // 16, 32, 64 or 128
+    return hp == 16 ? 4 : hp == 32 ? 5 : hp == 64 ? 6 : 7;
+}
+
+cudaError_t zero(float *p, size_t n, cudaStream_t s) {
+    return cudaMemsetAsync(p, 0, sizeof(float) * n, s);
 }
 
 template <class T>
 cudaError_t qkv_t(const Dims &dm, const void *X, const void *Wq, const void *Wk, const void *Wv,
                   const Saved &sv, cudaStream_t s) {
-    QkvOp<T> op{dm.B * dm.k, 3 * dm.hp, dm.d, dm.hp, (const T *)X, (const T *)Wq, (const T *)Wk,
+    QkvOp<T> op{dm.B * dm.k, 3 * dm.hp, dm.d, dm.hp, log2_of(dm.hp), (const T *)X, (const T *)Wq, (const T *)Wk,
                 (const T *)Wv, sv.gidx, sv.Q, sv.K, sv.V};
-    return launch_simt_gemm(op, dm.H, s);
+    op.lda = dm.d;
+    op.ldb = dm.hp;
+    return product(op, dm.H, 1, use_split() && aligned16({X, Wq, Wk, Wv}), sv, s);
 }
 
 template <class T>
 cudaError_t out_t(const Dims &dm, const void *Wo, const Saved &sv, float *Y, cudaStream_t s) {
     if (!dm.accumulate) {
-        cudaError_t e = cudaMemsetAsync(Y, 0, sizeof(float) * (size_t)dm.B * dm.T * dm.d, s);
+        const cudaError_t e = zero(Y, (size_t)dm.B * dm.T * dm.d, s);
         if (e != cudaSuccess) return e;
     }
-    OutOp<T> op{dm.B * dm.k, dm.d, dm.hp, sv.AR, (const T *)Wo, sv.gidx, Y};
-    return launch_simt_gemm(op, dm.H, s);
+    OutOp<T> op{dm.B * dm.k, dm.d, dm.hp, (const T *)sv.AR, (const T *)Wo, sv.gidx, Y};
+    op.lda = inter_ld<T>(dm.hp);
+    op.a_lo = dm.hp;
+    op.ldb = dm.d;
+    return product(op, dm.H, 1, use_split() && aligned16({Wo, Y}), sv, s);
 }
 
 template <class T>
 cudaError_t out_bwd_t(const Dims &dm, const void *Wo, const void *dY, const Saved &sv,
                       float *dWo, cudaStream_t s) {
-    OutBwdGOp<T> g{dm.B * dm.k, dm.hp, dm.d, (const T *)dY, (const T *)Wo, sv.gidx, sv.G};
-    cudaError_t e = launch_simt_gemm(g, dm.H, s);
+    using TS = typename InterOf<T>::type;
+    const bool split = use_split() && aligned16({Wo, dY, dWo});
+    const int Mtok = dm.B * dm.k;
+    OutBwdGOp<T> g{Mtok, dm.hp, dm.d, (const T *)dY, (const T *)Wo, sv.gidx, sv.G};
+    g.lda = dm.d;
+    g.ldb = dm.d;
+    cudaError_t e = product(g, dm.H, 1, split, sv, s);
     if (e != cudaSuccess) return e;
     const long long rows = dm.rows();
     const int warps = 8;
-    out_bwd_rows_kernel<typename InterOf<T>::type>
-        <<<(unsigned)((rows + warps - 1) / warps), warps * 32, 0, s>>>(
-            sv.G, sv.A, sv.rsel, sv.dA, sv.Dd, sv.dlogit, rows, dm.hp);
+    e = launch_pdl(out_bwd_rows_kernel<TS>, dim3((unsigned)((rows + warps - 1) / warps)),
+                   dim3(warps * 32), 0, s, (const float *)sv.G, (const float *)sv.A,
+                   (const float *)sv.rsel, sv.dA, sv.Dd, sv.dlogit, sv.dQKV, rows, dm.hp);
     note_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    OutBwdWOp<T> w{dm.hp, dm.d, dm.B * dm.k, sv.AR, (const T *)dY, sv.gidx, dWo};
-    return launch_simt_gemm(w, dm.H, s);
+    if (e != cudaSuccess) return e;
+    const int splits = split ? split_count(dm.d, dm.hp, Mtok, dm.H) : 1;
+    if (splits > 1 && (e = zero(dWo, (size_t)dm.H * dm.hp * dm.d, s)) != cudaSuccess) return e;
+    OutBwdWOp<T> w{dm.d, dm.hp, Mtok, (const T *)dY, (const T *)sv.AR, sv.gidx, dWo};
+    w.lda = dm.d;
+    w.ldb = inter_ld<T>(dm.hp);
+    w.b_lo = dm.hp;
+    return product(w, dm.H, splits, split, sv, s);
 }
 
 template <class T>
 cudaError_t in_bwd_t(const Dims &dm, const void *Wq, const void *Wk, const void *Wv,
                      const void *Wr, const Saved &sv, float *dX, cudaStream_t s) {
     if (!dm.accumulate) {
-        cudaError_t e = cudaMemsetAsync(dX, 0, sizeof(float) * (size_t)dm.B * dm.T * dm.d, s);
+        const cudaError_t e = zero(dX, (size_t)dm.B * dm.T * dm.d, s);
         if (e != cudaSuccess) return e;
     }
-    InBwdOp<T> op{dm.B * dm.k, dm.d, 3 * dm.hp, dm.hp, dm.H, sv.dQKV, (const T *)Wq,
+    InBwdOp<T> op{dm.B * dm.k, dm.d, 3 * dm.hp, dm.hp, log2_of(dm.hp), dm.H, (const T *)sv.dQKV, (const T *)Wq,
                   (const T *)Wk, (const T *)Wv, (const T *)Wr, sv.dlogit, sv.gidx, dX};
-    return launch_simt_gemm(op, dm.H, s);
+    op.lda = inter_ld<T>(4 * dm.hp);
+    op.a_lo = 4 * dm.hp;
+    op.ldb = dm.hp;
+    return product(op, dm.H, 1, use_split() && aligned16({Wq, Wk, Wv, dX}), sv, s);
 }
 
 template <class T>
 cudaError_t w_bwd_t(const Dims &dm, const void *X, const Saved &sv, float *dWq, float *dWk,
                     float *dWv, float *dWr, cudaStream_t s) {
-    WBwdOp<T> op{dm.d, 3 * dm.hp + 1, dm.B * dm.k, dm.hp, dm.H, (const T *)X,
-                 sv.dQKV, sv.dlogit, sv.gidx, dWq, dWk, dWv, dWr};
-    return launch_simt_gemm(op, dm.H, s);
+    const bool split = use_split() && aligned16({X, dWq, dWk, dWv});
+    const int N = 3 * dm.hp + WBwdOp<T>::kExtra, Mtok = dm.B * dm.k;
+    const int splits = split ? split_count(dm.d, N, Mtok, dm.H) : 1;
+    if (splits > 1) {
+        const size_t n = (size_t)dm.H * dm.d * dm.hp;
+        cudaError_t e;
+        if ((e = zero(dWq, n, s)) != cudaSuccess || (e = zero(dWk, n, s)) != cudaSuccess ||
+            (e = zero(dWv, n, s)) != cudaSuccess ||
+            (e = zero(dWr, (size_t)dm.d * dm.H, s)) != cudaSuccess)
+            return e;
+    }
+    WBwdOp<T> op{dm.d, N, Mtok, dm.hp, log2_of(dm.hp), dm.H, (const T *)X, (const T *)sv.dQKV, sv.dlogit, sv.gidx,
+                 dWq, dWk, dWv, dWr};
+    op.lda = dm.d;
+    op.ldb = inter_ld<T>(4 * dm.hp);
+    op.b_lo = 4 * dm.hp;
+    return product(op, dm.H, splits, split, sv, s);
 }
 
 }  // namespace
 
-bool use_tc(const Dims &dm) {
+bool use_split() {
     const char *f = std::getenv("MOSA_FORCE_SIMT");
-    if (f != nullptr && f[0] != '\0' && f[0] != '0') return false;
-    return tc_supported(dm);
+    return f == nullptr || f[0] == '\0' || f[0] == '0';
 }
+
+bool use_tc(const Dims &dm) { return use_split() && tc_supported(dm); }
 
 bool use_fused_forward(const Dims &dm) {
     const char *f = std::getenv("MOSA_FUSED_FWD");
