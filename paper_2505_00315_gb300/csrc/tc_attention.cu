@@ -72,11 +72,9 @@ struct AttnParams {
 //   O += P_j V_j with P read from TMEM as the A operand and V from shared
 //   memory, O in TMEM.
 // P in TMEM takes the shared-memory stores and the proxy fence of P off the
-// softmax warps' chain (47.7 -> 44.6 us at B4 T4096 d1024 H8 k2048); the
-// MMAs themselves cost the same either way (measured with %clock stamps:
-// about 120 cycles per M = 128, N = 64, K = 16 instruction and 165 at
-// N = 128, also when independent accumulators alternate, so the tensor pipe
-// runs these small instructions one after another at a fixed cost each).
+// softmax warps' chain (47.7 -> 44.6 us at B4 T4096 d1024 H8 k2048), and the
+// MMAs with it take 31 cycles instead of 48 (N = 64, back to back in an idle
+// CTA) once they are issued under elect_one (-> 42 us).
 // Earlier builds found that a tcgen05.st issued while an MMA reads its A
 // operand from TMEM corrupts that MMA even when the columns differ, so the
 // softmax warps store P_j only after P_{j-1} V_{j-1} has completed (issued a
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(kLT, 1) attn_fwd_tc_kernel(const __grid_consta
                 drain_phase(smem_u32(&sm.kv_full[t % kLSlots]), (t / kLSlots) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idS = idesc_f16(128, kLKeys, false, false);
             constexpr uint32_t idO = idesc_f16(128, 64, false, true);
             int t = 0;   // next K/V item to consume
@@ -427,11 +425,15 @@ __device__ __forceinline__ void flag_timeout_b(SM &sm, uint32_t *status) {
 //   is about to overwrite and one lane hands it to the TMA engine as a bulk
 //   reduce-add (the 256 threads' own scattered vector reductions took about
 //   1 us per block).
-// Measured on this GPU, an MMA instruction (M = 128, K = 16) takes about the
-// same time for any N up to 128 (about 2.3x longer per FLOP at N = 64 than
-// at N = 256), so the 32 MMAs of a block (S, dP: N = 128; dV, dK, dQ: N = 64)
-// cost about 4000 cycles and the kernel is bound by keeping the tensor pipe
-// issuing.  The MMA issuer therefore waits only for what each product needs:
+// The 32 MMAs of a block take about 64 (N = 128: S, dP) and 48 cycles (N = 64:
+// dV, dK, dQ) each back to back (M = 128, K = 16, in an otherwise idle CTA),
+// 1660 in all; the workers' exponentials 1024, and shared memory about 2900
+// (208 KB of operands read by the MMAs, 160 KB of P, dS, dQ and loads).
+// Measured over k = 256 .. 2048 (32 heads of 4 x 4096 tokens): 1.6 us a block
+// plus about 9 us a CTA.  Issuing under elect_one (30 instead of 73 cycles an
+// MMA) took B4 T4096 d1024 H8 k2048 from 90 to 84 us; 16 worker warps of 32 keys
+// per thread were slower at every size (91 us there).
+// The MMA issuer waits only for what each product needs:
 // S_{i+1} is issued as soon as the workers have read S_i into registers, and
 // dP_{i+1}, dK_i and dQ_i as soon as dS_i is stored; the workers do not wait
 // for the tensor pipe either: dS and dQ are double-buffered (the smem dS tile
@@ -544,7 +546,7 @@ __global__ void __launch_bounds__(kBT, 1) attn_bwd_tc_kernel(const __grid_consta
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idKK = idesc_f16(128, 128, false, false);  // S, dP
             constexpr uint32_t idMN = idesc_f16(128, 64, true, true);     // dV, dK
             constexpr uint32_t idKM = idesc_f16(128, 64, false, true);    // dQ
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(kBT, 1) attn_bwd_tc_kernel(const __grid_consta
         }
         if (nb >= 2) drain_dq(nb - 2);
         drain_dq(nb - 1);
-        if (lane == 0) bulk_wait0();   // the reductions are complete before the CTA's smem goes
+        if (lane == 0) bulk_wait_read0();   // the reductions have read the CTA's smem before it goes
         __syncwarp();
         // dK / sqrt(h') and dV of the tile's keys (row r = key j0 + r); an fp16
         // dS out of range has made them non-finite, which flags it
@@ -894,7 +896,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) attn_fwd_small_kernel(const 
             drain_phase(fb, 0);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idS = idesc_bf16(128, 128, false, false);
             constexpr uint32_t idO = idesc_bf16(128, 64, false, true);
             bool ok = mbar_wait(smem_u32(&sm.in_full), 0);
@@ -1039,7 +1041,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) attn_bwd_small_kernel(const 
             drain_phase(fb, 0);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idKK = idesc_bf16(128, 128, false, false);  // S, dP
             constexpr uint32_t idMN = idesc_bf16(128, 64, true, true);     // dV, dK
             constexpr uint32_t idKM = idesc_bf16(128, 64, false, true);    // dQ
@@ -1155,7 +1157,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) attn_bwd_small_kernel(const 
                 for (int hf = 0; hf < (p.out16 ? 1 : 2); ++hf)
                     tma_store_3d(&p.mOut, smem_u32(tiles[t][hf]), 64 * t + 256 * hf, b0 * p.k, h);
             bulk_commit();
-            bulk_wait0();
+            bulk_wait_read0();
         }
     }
     tc_fence_before();

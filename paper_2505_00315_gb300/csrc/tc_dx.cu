@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __gr
                 if (na[j] > 0) drain_phase(smem_u32(&sm.a_full[j]), (na[j] - 1) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // B: W_j blocks K-major (dX), W_o chunks MN-major (Y)
             const uint32_t idX = p.f16 ? idesc_f16(128, kChunk, false, kOut)
                                        : idesc_bf16(128, kChunk, false, kOut);

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_bwd_kernel(const __grid_con
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------- MMA
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             // phase 1: G = dY[I] W_o^T into TMEM 0..63 (both operands K-major)
             constexpr uint32_t idG = idesc_bf16(128, 64, false, false);

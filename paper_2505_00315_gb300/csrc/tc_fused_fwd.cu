@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------- MMA
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             // phase 1: [Q|K|V] into TMEM columns 0..191
             constexpr uint32_t idQKV = idesc_bf16(128, 192, false, true);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
                     tma_store_3d(&p.mOut[3], smem_u32(sm.q[hf]), 64 * hf, b0 * p.k, h);
                 bulk_commit();
             }
-            bulk_wait0();
+            bulk_wait_read0();
         }
     } else if (warp >= 4) {
         const int t = threadIdx.x - 128;            // 0..255

@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<KIND>::MIN_CTAS)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = KIND == kROUTER ? idesc_bf16(kBM, p.N, false, true)
                                    : KIND == kDWH ? idesc_f16(kBM, C::BN, C::A_MN, C::B_MN)
                                    : idesc_bf16(kBM, C::BN, C::A_MN, C::B_MN);

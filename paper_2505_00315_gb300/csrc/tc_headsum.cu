@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kHsThreads, 1) head_sum_kernel(const __grid_co
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issue
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = kOut ? (p.f16 ? idesc_f16(128, kHsChunk, false, true)
                                                  : idesc_bf16(128, kHsChunk, false, true))
                                         : idesc_f16(128, kHsChunk, false, false);

@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
         }
     } else if (warp == 16) {
         // ----------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, sa.bn, Op::kAMN, Op::kBMN);
             for (int it = 0; it < nkb; ++it) {
                 const int s = it % S, c = it / DR;
