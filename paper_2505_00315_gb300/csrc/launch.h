@@ -18,26 +18,41 @@ namespace mosa {
 // A kernel that shares the GPU with another stream's kernel is launched late
 // instead: waiting early, its CTAs would hold SMs the other kernel needs.
 // MOSA_PDL=0 launches every kernel plainly.
+// priority (when not 0): the launch's scheduling priority, lower is sooner.
 template <class... KArgs, class... Args>
-inline cudaError_t launch_ex(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block,
-                             size_t smem, cudaStream_t s, Args &&...args) {
+inline cudaError_t launch_ex(bool early, int priority, void (*kernel)(KArgs...), dim3 grid,
+                             dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
     const char *v = std::getenv("MOSA_PDL");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = (!early || (v != nullptr && v[0] == '0')) ? 0 : 1;
+    if (early && (v == nullptr || v[0] != '0')) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (priority != 0) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePriority;
+        attr[cfg.numAttrs++].val.priority = priority;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, Args &&...args) {
-    return launch_ex(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
+    return launch_ex(true, 0, kernel, grid, block, smem, s, std::forward<Args>(args)...);
+}
+// As launch_pdl, ahead of the side stream's copies and zeroing: the kernels that
+// follow TopK on the caller's stream (the greatest priority of the device).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_ahead(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t s, Args &&...args) {
+    int least = 0, greatest = 0;
+    (void)cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    return launch_ex(true, greatest, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 
 // Raises `kernel`'s dynamic shared-memory limit to `bytes` on the current
@@ -191,9 +206,8 @@ cudaError_t tc_dx(const Dims &dm, const void *Wq, const void *Wk, const void *Wv
 bool tc_router_applies(const Dims &dm);
 bool tc_router(const Dims &dm, const void *X, const void *Wr, int wr_cols, float *r_full,
                uint32_t *status, cudaStream_t s, cudaError_t *err);
-// bf16 -> fp16 copy of n values (n % 8 == 0, 16-byte aligned); values beyond
-// the fp16 range set kStatusRange.
-cudaError_t tc_to_f16(const void *src, void *dst, size_t n, uint32_t *status, cudaStream_t s);
+// Zeroes n fp32 values in short CTAs (see to_f16_kernel).
+cudaError_t launch_zero(float *p, size_t n, cudaStream_t s);
 // Address of the fp16 copy of W_o inside sv.W16.
 void *wo16_of(const Dims &dm, const Saved &sv);
 // fp16 attention path: X -> sv.X16 and W_q, W_k, W_v, W_o -> sv.W16 (bf16 ->

@@ -122,16 +122,26 @@ struct DevResources {
     cudaEvent_t ev[4] = {};
 };
 constexpr int kMaxDev = 64;
+constexpr int kMaxPrio = 8;   // stream priorities 0, -1, ..
 std::mutex g_res_mu;
-DevResources g_res[kMaxDev];
+DevResources g_res[kMaxDev][kMaxPrio];
 
-DevResources *dev_resources() {
+// Priority of the caller's stream as an index 0 .. kMaxPrio - 1 (0: the default).
+// Layer graphs run by the priorities of their nodes (cudaGraphInstantiateFlagUseNodePriority),
+// so the internal streams a call is captured on take the caller's.
+int priority_index(cudaStream_t s) {
+    int prio = 0;
+    if (cudaStreamGetPriority(s, &prio) != cudaSuccess) return 0;
+    return prio >= 0 ? 0 : (-prio < kMaxPrio ? -prio : kMaxPrio - 1);
+}
+
+DevResources *dev_resources(int prio) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return nullptr;
     std::lock_guard<std::mutex> lk(g_res_mu);
-    DevResources &r = g_res[dev];
+    DevResources &r = g_res[dev][prio];
     if (r.side == nullptr) {
-        if (cudaStreamCreateWithFlags(&r.side, cudaStreamNonBlocking) != cudaSuccess) {
+        if (cudaStreamCreateWithPriority(&r.side, cudaStreamNonBlocking, -prio) != cudaSuccess) {
             r.side = nullptr;
             return nullptr;
         }
@@ -202,7 +212,7 @@ mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const voi
     MOSA_TRY(link(s, r.side, r.ev[0]));
     // (the token-major output product writes every element of Y itself)
     const bool headsum = !use_fused_forward(dm) && use_headsum_out(dm);
-    if (!dm.accumulate && !headsum) MOSA_TRY(cudaMemsetAsync(Y, 0, sizeof(float) * ny, r.side));
+    if (!dm.accumulate && !headsum) MOSA_TRY(launch_zero(Y, ny, r.side));
     // the fused k <= 128 kernel needs only Y zeroed from the side stream
     const bool fused = use_fused_forward(dm);
     if (fused) MOSA_TRY(cudaEventRecord(r.ev[1], r.side));
@@ -507,7 +517,7 @@ mosa_status check_hybrid_workspace(const Hybrid &h, void *ws, size_t bytes, Hybr
 // graph on the caller's stream.  MOSA_GRAPHS=0 turns this off.
 
 struct GraphKey {
-    int op, device, tc;
+    int op, device, tc, prio;
     uint32_t mask;
     mosa_shape shape;
     int extra[2];  // hybrid calls: dense heads, window
@@ -530,10 +540,9 @@ struct GraphEntry {
 };
 
 constexpr size_t kMaxGraphs = 128;
-constexpr int kMaxDevices = 64;
 std::mutex g_graph_mu;
 std::unordered_map<GraphKey, GraphEntry *, GraphKeyHash> g_graphs;
-cudaStream_t g_capture_stream[kMaxDevices] = {};
+cudaStream_t g_capture_stream[kMaxDev][kMaxPrio] = {};
 
 bool graphs_enabled() {
     const char *v = std::getenv("MOSA_GRAPHS");
@@ -545,12 +554,13 @@ int path_bits(const Dims &dm) {
            (use_headsum_out(dm) ? 8 : 0) | (use_headsum_dx(dm) ? 16 : 0) | (use_split() ? 32 : 0);
 }
 
-GraphKey make_key(int op, const Dims &dm, const mosa_shape *shape,
+GraphKey make_key(int op, int prio, const Dims &dm, const mosa_shape *shape,
                   std::initializer_list<const void *> ptrs, const Dims *dense = nullptr,
                   int extra0 = 0, int extra1 = 0) {
     GraphKey k;
     std::memset(&k, 0, sizeof(k));
     k.op = op;
+    k.prio = prio;
     cudaGetDevice(&k.device);
     k.tc = path_bits(dm) | (dense ? path_bits(*dense) << 6 : 0);
     k.mask = profile_mask();
@@ -568,13 +578,14 @@ mosa_status run_graphed(const GraphKey &key, cudaStream_t user, Enqueue &&enqueu
     // One lock for both paths: the eager path shares the internal side stream
     // and its events between calls.
     std::lock_guard<std::mutex> lk(g_graph_mu);
-    if (!graphs_enabled() || key.device < 0 || key.device >= kMaxDevices) return enqueue(user);
+    if (!graphs_enabled() || key.device < 0 || key.device >= kMaxDev) return enqueue(user);
     auto it = g_graphs.find(key);
     GraphEntry *e = it == g_graphs.end() ? nullptr : it->second;
     if (e == nullptr) {
         if (g_graphs.size() >= kMaxGraphs) return enqueue(user);
-        cudaStream_t &cs = g_capture_stream[key.device];
-        if (cs == nullptr && cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaStream_t &cs = g_capture_stream[key.device][key.prio];
+        if (cs == nullptr &&
+            cudaStreamCreateWithPriority(&cs, cudaStreamNonBlocking, -key.prio) != cudaSuccess) {
             cs = nullptr;
             return enqueue(user);
         }
@@ -587,7 +598,8 @@ mosa_status run_graphed(const GraphKey &key, cudaStream_t user, Enqueue &&enqueu
             if (cudaStreamEndCapture(cs, &g) != cudaSuccess) st = MOSA_ERR_CUDA;
         }
         capture_into(nullptr);
-        if (st == MOSA_OK && g != nullptr && cudaGraphInstantiate(&e->exec, g, 0) != cudaSuccess)
+        if (st == MOSA_OK && g != nullptr &&
+            cudaGraphInstantiate(&e->exec, g, cudaGraphInstantiateFlagUseNodePriority) != cudaSuccess)
             st = MOSA_ERR_CUDA;
         if (g != nullptr) cudaGraphDestroy(g);
         if (st != MOSA_OK) {
@@ -651,11 +663,12 @@ mosa_status mosa_forward(const mosa_shape *shape, const void *X, const void *W_r
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sv.r_full;
-    DevResources *res = use_tc(dm) ? dev_resources() : nullptr;
+    const int prio = priority_index((cudaStream_t)stream);
+    DevResources *res = use_tc(dm) ? dev_resources(prio) : nullptr;
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         return forward_routed(dm, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf, sv, s, res);
     };
-    const GraphKey key = make_key(0, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, r_full,
+    const GraphKey key = make_key(0, prio, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, r_full,
                                                  workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
@@ -670,11 +683,12 @@ mosa_status mosa_forward_with_indices(const mosa_shape *shape, const void *X, co
     if (!X || !W_q || !W_k || !W_v || !W_o || !I || !r_sel || !Y) return MOSA_ERR_INVALID_ARG;
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
-    DevResources *res = use_tc(dm) ? dev_resources() : nullptr;
+    const int prio = priority_index((cudaStream_t)stream);
+    DevResources *res = use_tc(dm) ? dev_resources(prio) : nullptr;
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         return forward_given(dm, X, W_q, W_k, W_v, W_o, I, r_sel, Y, sv, s, res);
     };
-    const GraphKey key = make_key(1, dm, shape, {X, W_q, W_k, W_v, W_o, I, r_sel, Y, workspace});
+    const GraphKey key = make_key(1, prio, dm, shape, {X, W_q, W_k, W_v, W_o, I, r_sel, Y, workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
 
@@ -691,12 +705,13 @@ mosa_status mosa_backward(const mosa_shape *shape, const void *X, const void *W_
         return MOSA_ERR_INVALID_ARG;
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
-    DevResources *res = use_tc(dm) ? dev_resources() : nullptr;
+    const int prio = priority_index((cudaStream_t)stream);
+    DevResources *res = use_tc(dm) ? dev_resources(prio) : nullptr;
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         return backward_all(dm, X, W_r, W_q, W_k, W_v, W_o, dY, dX, dW_r, dW_q, dW_k, dW_v, dW_o,
                             sv, s, res);
     };
-    const GraphKey key = make_key(2, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, I, r_sel, dY, dX,
+    const GraphKey key = make_key(2, prio, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, I, r_sel, dY, dX,
                                                  dW_r, dW_q, dW_k, dW_v, dW_o, workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
@@ -722,15 +737,16 @@ mosa_status mosa_hybrid_forward(const mosa_hybrid_shape *shape, const void *X, c
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sp.sparse.r_full;
-    DevResources *rs = use_tc(h.sparse) ? dev_resources() : nullptr;
-    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources() : nullptr;
+    const int prio = priority_index((cudaStream_t)stream);
+    DevResources *rs = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
+    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources(prio) : nullptr;
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         mosa_status e = forward_routed(h.sparse, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf,
                                        sp.sparse, s, rs);
         if (e != MOSA_OK || !h.has_dense) return e;
         return forward_given(h.dense, X, D_q, D_k, D_v, D_o, nullptr, nullptr, Y, sp.dense, s, rd);
     };
-    const GraphKey key = make_key(3, h.sparse, &shape->sparse,
+    const GraphKey key = make_key(3, prio, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, Y, I, r_sel,
                                    r_full, workspace},
                                   h.has_dense ? &h.dense : nullptr, shape->H_dense, shape->window);
@@ -755,8 +771,9 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
         return MOSA_ERR_INVALID_ARG;
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
-    DevResources *rs = use_tc(h.sparse) ? dev_resources() : nullptr;
-    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources() : nullptr;
+    const int prio = priority_index((cudaStream_t)stream);
+    DevResources *rs = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
+    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources(prio) : nullptr;
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         mosa_status e = backward_all(h.sparse, X, W_r, W_q, W_k, W_v, W_o, dY, dX, dW_r, dW_q,
                                      dW_k, dW_v, dW_o, sp.sparse, s, rs);
@@ -765,7 +782,7 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
         return backward_all(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q,
                             dD_k, dD_v, dD_o, sp.dense, s, rd);
     };
-    const GraphKey key = make_key(4, h.sparse, &shape->sparse,
+    const GraphKey key = make_key(4, prio, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, I, r_sel, dY,
                                    dX, dW_r, dW_q, dW_k, dW_v, dW_o, dD_q, dD_k, dD_v, dD_o,
                                    workspace},

@@ -491,7 +491,7 @@ cudaError_t launch_select(int rows, int T, int k, const float *scores, int32_t *
     // 4096, 512 and 1024 x 4096, 64 x 8192)
     int threads = T / 4 < 256 ? 256 : (T / 4 > 1024 ? 1024 : (T / 4 + 31) / 32 * 32);
     if (rows >= 512 && threads > 512) threads = 512;
-    cudaError_t e = launch_pdl(topk_select_kernel, dim3(rows), dim3(threads), smem, stream,
+    cudaError_t e = launch_ahead(topk_select_kernel, dim3(rows), dim3(threads), smem, stream,
                                scores, T, k, I, rsel, B, H, gidx, rsel_hm, first_token ? 1 : 0,
                                active_span());
     note_launches(1);

@@ -482,7 +482,7 @@ cudaError_t tc_fused_forward(const Dims &dm, const void *X, const void *Wq, cons
     const cudaError_t attr = allow_smem((const void *)fused_fwd_kernel, kSmem);
     if (attr != cudaSuccess) return attr;
     const dim3 grid((dm.B + p.U - 1) / p.U, dm.H);
-    cudaError_t e = launch_pdl(fused_fwd_kernel, grid, dim3(kThreads), kSmem, s, p);
+    cudaError_t e = launch_ahead(fused_fwd_kernel, grid, dim3(kThreads), kSmem, s, p);
     note_launches(1);
     return e;
 }

@@ -840,12 +840,14 @@ bool map_heads(CUtensorMap *m, const void *base, uint64_t H, uint64_t rows, uint
 }
 
 template <int KIND>
-cudaError_t launch_kind(const TcParams &p, dim3 grid, cudaStream_t s, bool early = true) {
+cudaError_t launch_kind(const TcParams &p, dim3 grid, cudaStream_t s) {
     constexpr int smem = smem_bytes<KIND>();
     if (p.wait_ns == 0) return cudaErrorInvalidValue;  // every launcher sets a wait limit
     const cudaError_t attr = allow_smem((const void *)tc_gemm_kernel<KIND>, smem);
     if (attr != cudaSuccess) return attr;
-    cudaError_t e = launch_ex(early, tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p);
+    cudaError_t e = KIND == kQKV
+                        ? launch_ahead(tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p)
+                        : launch_pdl(tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p);
     note_launches(1);
     return e;
 }
@@ -917,17 +919,35 @@ bool tc_router(const Dims &dm, const void *X, const void *Wr, int wr_cols, float
     return true;
 }
 
-// bf16 -> fp16, eight values per 16-byte step (bf16x8_to_f16x8); a value
-// beyond the fp16 range sets kStatusRange.
-__global__ void to_f16_kernel(const uint4 *__restrict__ src, uint4 *__restrict__ dst, size_t n8,
-                              uint32_t *status) {
-    pdl_wait();
-    pdl_trigger();
+// Side-stream work of the forward: the fp16 copies (bf16x8_to_f16x8; a value
+// beyond the fp16 range sets kStatusRange) and zeroing.  Each CTA of 256
+// threads handles one 16-byte unit per thread and ends, so that TopK and the
+// kernel after it, launched ahead of these in priority, get an SM as soon as a few
+// of them have ended: with grid-stride CTAs over whole copies the kernel after TopK
+// waited until the copies were through (16 us at B16 T1024 d1024 H64 k64, whose
+// step went from 375 to 365 us; B2 T8192 d1024 H32 k256 168.5 -> 164; four
+// units per thread in flight slowed TopK: 371 and 166).
+constexpr int kSideCta = 256;   // units per CTA
+
+struct F16Copies {
+    const uint4 *src[5];
+    uint4 *dst[5];
+    size_t n8[5];        // units of each array
+    unsigned cta0[6];    // first CTA of each array; cta0[5]: all of them
+};
+
+__global__ void __launch_bounds__(kSideCta) to_f16_kernel(const F16Copies c, uint32_t *status) {
+    int a = 0;
+    while (blockIdx.x >= c.cta0[a + 1]) ++a;
+    const size_t i = (size_t)(blockIdx.x - c.cta0[a]) * kSideCta + threadIdx.x;
     bool bad = false;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8;
-         i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = bf16x8_to_f16x8(src[i], bad);
+    if (i < c.n8[a]) c.dst[a][i] = bf16x8_to_f16x8(c.src[a][i], bad);
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kStatusRange);
+}
+
+__global__ void __launch_bounds__(kSideCta) zero_kernel(float4 *p, size_t n4) {
+    const size_t i = (size_t)blockIdx.x * kSideCta + threadIdx.x;
+    if (i < n4) p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 __global__ void transpose_wr_kernel(const bf16 *__restrict__ Wr, float *__restrict__ WrT, int d,
@@ -940,12 +960,12 @@ __global__ void transpose_wr_kernel(const bf16 *__restrict__ Wr, float *__restri
     }
 }
 
-cudaError_t tc_to_f16(const void *src, void *dst, size_t n, uint32_t *status, cudaStream_t s) {
-    const size_t n8 = n / 8;
-    if (n8 == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)std::min<size_t>((n8 + 255) / 256, 1216);
-    to_f16_kernel<<<grid, 256, 0, s>>>(static_cast<const uint4 *>(src), static_cast<uint4 *>(dst),
-                                       n8, status);
+cudaError_t launch_zero(float *p, size_t n, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    if (n % 4 != 0 || (reinterpret_cast<uintptr_t>(p) & 15) != 0)
+        return cudaMemsetAsync(p, 0, sizeof(float) * n, s);
+    zero_kernel<<<(unsigned)((n / 4 + kSideCta - 1) / kSideCta), 256, 0, s>>>(
+        reinterpret_cast<float4 *>(p), n / 4);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -961,12 +981,22 @@ cudaError_t tc_f16_copies(const Dims &dm, const void *X, const void *Wq, const v
     void *dst[5] = {sv.X16, sv.W16, (char *)sv.W16 + 2 * nw, (char *)sv.W16 + 4 * nw,
                     wo16_of(dm, sv)};
     const size_t n[5] = {(size_t)dm.B * dm.T * dm.d, nw, nw, nw, nw};   // d % 8 == 0
+    F16Copies c = {};
+    int m = 0;
+    unsigned ctas = 0;
     for (int i = 0; i < 5; ++i) {
-        if (src[i] == nullptr) continue;
-        const cudaError_t e = tc_to_f16(src[i], dst[i], n[i], sv.status, s);
-        if (e != cudaSuccess) return e;
+        if (src[i] == nullptr || n[i] == 0) continue;
+        c.src[m] = static_cast<const uint4 *>(src[i]);
+        c.dst[m] = static_cast<uint4 *>(dst[i]);
+        c.n8[m] = n[i] / 8;
+        c.cta0[m++] = ctas;
+        ctas += (unsigned)((n[i] / 8 + kSideCta - 1) / kSideCta);
     }
-    return cudaSuccess;
+    if (ctas == 0) return cudaSuccess;
+    for (; m < 6; ++m) c.cta0[m] = ctas;
+    to_f16_kernel<<<ctas, 256, 0, s>>>(c, sv.status);
+    note_launches(1);
+    return cudaGetLastError();
 }
 
 cudaError_t tc_transpose_wr(const Dims &dm, const void *Wr, const Saved &sv, cudaStream_t s) {
