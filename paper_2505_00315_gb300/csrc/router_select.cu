@@ -39,23 +39,32 @@ struct RouterOp {
 };
 
 // Router on CUDA cores (fp32 storage, and bf16 where the tensor-core router does
-// not apply: H % 8 != 0 or a head size other than 64).  A CTA of 128 threads
-// computes 32 tokens x HT heads (HT = 16, 32 or 64), HT/16 x 4 per thread, each
+// not apply: H % 8 != 0 or a head size other than 64).  A CTA computes 32 or (HT =
+// 64) 64 tokens x HT heads (HT = 16, 32 or 64), HT/16 x 4 per thread, each
 // score one multiply-add chain over d in ascending order (so that the scores
 // do not depend on HT, and match RouterOp's bit for bit).  X comes through a
-// ring of kRouterStages chunks of 2048 / HT columns by 16-byte cp.async and is
+// ring of kRouterStages chunks of KC columns by 16-byte cp.async and is
 // read eight columns of a token at a time; W_r (rows of any alignment) goes through
-// registers, one chunk ahead, into an fp32 tile.  Measured alone: B4 T2048
-// d1024 H60 193 us with the general 64 x 64 tile product (scalar loads, nothing
-// in flight across its barriers), 48 us now; B1 T1531 d768 H12 129 -> 14 us;
-// fp32 B4 T1000 d768 H12 152 -> 14 us.
-constexpr int kRouterThreads = 128, kRouterTok = 32, kRouterElems = 2048, kRouterStages = 4;
+// registers, 16 elements per thread, one chunk ahead, into an fp32 tile.  Measured
+// alone: B4 T2048 d1024 H60 193 us with the general 64 x 64 tile product (scalar
+// loads, nothing in flight across its barriers), 42 us now, bound by its issue
+// slots (80% of them used, 60% of those by the multiply-adds; packed
+// fma.rn.f32x2 on X converted in shared memory was slower, 46 us); B1 T1531 d768
+// H12 129 -> 12 us; fp32 B4 T1000 d768 H12 152 -> 14 us.
+constexpr int kRouterStages = 4;
+template <int HT>
+struct RouterTile {
+    static constexpr int THREADS = HT == 64 ? 256 : 128, TOK = THREADS / 4;
+    static constexpr int ELEMS = 16 * THREADS;   // of W_r per chunk
+    static constexpr int KC = ELEMS / HT;        // columns of d per chunk
+};
 
 template <class E, int HT>
-constexpr int router_ld() { return kRouterElems / HT + 16 / (int)sizeof(E); }   // X row stride
+constexpr int router_ld() { return RouterTile<HT>::KC + 16 / (int)sizeof(E); }   // X row stride
 template <class E, int HT>
 constexpr int router_smem() {
-    return kRouterElems * 4 + kRouterStages * kRouterTok * router_ld<E, HT>() * (int)sizeof(E);
+    return RouterTile<HT>::ELEMS * 4 +
+           kRouterStages * RouterTile<HT>::TOK * router_ld<E, HT>() * (int)sizeof(E);
 }
 
 // Eight consecutive elements as fp32.
@@ -74,21 +83,22 @@ __device__ __forceinline__ void widen8(const bf16 *p, float (&v)[8]) {
 }
 
 template <class E, int HT>
-__global__ void __launch_bounds__(kRouterThreads)
+__global__ void __launch_bounds__(RouterTile<HT>::THREADS)
     router_rows_kernel(const E *__restrict__ X, const E *__restrict__ Wr, float *__restrict__ r_full,
                        int M, int T, int H, int d) {
-    constexpr int KC = kRouterElems / HT;          // columns of d per chunk
+    constexpr int THREADS = RouterTile<HT>::THREADS, TOK = RouterTile<HT>::TOK;
+    constexpr int KC = RouterTile<HT>::KC;
     constexpr int TM = HT / 16;                    // tokens per thread
     constexpr int UE = 16 / (int)sizeof(E);        // elements of a 16-byte unit
-    constexpr int UNITS = kRouterTok * KC / UE / kRouterThreads;   // X units per thread and chunk
-    constexpr int WV = kRouterElems / kRouterThreads;
+    constexpr int UNITS = TOK * KC / UE / THREADS; // X units per thread and chunk
+    constexpr int WV = RouterTile<HT>::ELEMS / THREADS;
     constexpr int XLD = router_ld<E, HT>(), S = kRouterStages;
     extern __shared__ __align__(16) uint8_t router_sm[];
     float *Ws = reinterpret_cast<float *>(router_sm);
-    E *Xs = reinterpret_cast<E *>(router_sm + kRouterElems * 4);
+    E *Xs = reinterpret_cast<E *>(router_sm + RouterTile<HT>::ELEMS * 4);
     const int tid = threadIdx.x;
     const int hg = tid % (HT / 4), tg = tid / (HT / 4);
-    const int m0 = blockIdx.x * kRouterTok, h0 = blockIdx.y * HT;
+    const int m0 = blockIdx.x * TOK, h0 = blockIdx.y * HT;
     const int chunks = (d + KC - 1) / KC;
     E wr[WV];
     float acc[TM][4];
@@ -97,10 +107,10 @@ __global__ void __launch_bounds__(kRouterThreads)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     auto fetch_x = [&](int c) {   // zeros past M and d (d % 8 == 0)
-        E *dst = Xs + (c % S) * kRouterTok * XLD;
+        E *dst = Xs + (c % S) * TOK * XLD;
 #pragma unroll
         for (int v = 0; v < UNITS; ++v) {
-            const int u = tid + kRouterThreads * v, tok = u / (KC / UE), q = u % (KC / UE);
+            const int u = tid + THREADS * v, tok = u / (KC / UE), q = u % (KC / UE);
             const int kx = c * KC + q * UE;
             const bool on = m0 + tok < M && kx < d;
             tc::cp_async16(tc::smem_u32(dst + tok * XLD + q * UE),
@@ -110,7 +120,7 @@ __global__ void __launch_bounds__(kRouterThreads)
     auto load_w = [&](int c) {
 #pragma unroll
         for (int v = 0; v < WV; ++v) {
-            const int e = tid + kRouterThreads * v, kx = c * KC + e / HT, h = h0 + e % HT;
+            const int e = tid + THREADS * v, kx = c * KC + e / HT, h = h0 + e % HT;
             wr[v] = kx < d && h < H ? Wr[(size_t)kx * H + h] : from_f32<E>(0.f);
         }
     };
@@ -123,13 +133,13 @@ __global__ void __launch_bounds__(kRouterThreads)
         tc::cp_async_wait<S - 2>();
         __syncthreads();   // chunk c of X is in; chunk c - 1 has been read
 #pragma unroll
-        for (int v = 0; v < WV; ++v) Ws[tid + kRouterThreads * v] = to_f32(wr[v]);
+        for (int v = 0; v < WV; ++v) Ws[tid + THREADS * v] = to_f32(wr[v]);
         if (c + S - 1 < chunks) fetch_x(c + S - 1);
         tc::cp_async_commit();
         __syncthreads();
         if (c + 1 < chunks) load_w(c + 1);
-        const E *xs = Xs + (c % S) * kRouterTok * XLD + tg * TM * XLD;
-#pragma unroll 2
+        const E *xs = Xs + (c % S) * TOK * XLD + tg * TM * XLD;
+#pragma unroll(TM == 4 ? 2 : 4)
         for (int k8 = 0; k8 < KC; k8 += 8) {
             float a[TM][8];
 #pragma unroll
@@ -151,7 +161,7 @@ __global__ void __launch_bounds__(kRouterThreads)
     // scores through shared memory, so that a warp writes 32 consecutive tokens
     tc::cp_async_wait<0>();
     __syncthreads();
-    constexpr int RLD = kRouterTok + 1;
+    constexpr int RLD = TOK + 1;
     float *Rs = Ws;
     static_assert(router_smem<E, HT>() >= HT * RLD * 4, "score tile must fit in the operand tiles");
 #pragma unroll
@@ -160,11 +170,11 @@ __global__ void __launch_bounds__(kRouterThreads)
         for (int j = 0; j < 4; ++j)
             Rs[(4 * hg + j) * RLD + tg * TM + i] = 1.f / (1.f + expf(-acc[i][j]));
     __syncthreads();
-    const int m = m0 + (tid & 31);
+    const int m = m0 + tid % TOK;
     if (m < M) {
         const int bb = m / T, t = m - bb * T;
-        for (int h = tid >> 5; h < HT && h0 + h < H; h += kRouterThreads / 32)
-            r_full[((size_t)bb * H + h0 + h) * T + t] = Rs[h * RLD + (tid & 31)];
+        for (int h = tid / TOK; h < HT && h0 + h < H; h += THREADS / TOK)
+            r_full[((size_t)bb * H + h0 + h) * T + t] = Rs[h * RLD + tid % TOK];
     }
 }
 
@@ -406,11 +416,12 @@ template <class E, int HT>
 static cudaError_t router_rows(const Dims &dm, const void *X, const void *Wr, float *r_full,
                                cudaStream_t stream) {
     const int M = dm.B * dm.T;
-    const dim3 grid((M + kRouterTok - 1) / kRouterTok, (dm.H + HT - 1) / HT);
+    constexpr int tok = RouterTile<HT>::TOK;
+    const dim3 grid((M + tok - 1) / tok, (dm.H + HT - 1) / HT);
     constexpr int smem = router_smem<E, HT>();
     const cudaError_t e = allow_smem((const void *)router_rows_kernel<E, HT>, smem);
     if (e != cudaSuccess) return e;
-    router_rows_kernel<E, HT><<<grid, kRouterThreads, smem, stream>>>(
+    router_rows_kernel<E, HT><<<grid, RouterTile<HT>::THREADS, smem, stream>>>(
         (const E *)X, (const E *)Wr, r_full, M, dm.T, dm.H, dm.d);
     note_launches(1);
     return cudaGetLastError();
