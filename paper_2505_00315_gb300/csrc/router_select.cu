@@ -1,16 +1,11 @@
 // Router (F1) and TopK selection (F2) of the MoSA layer, Sec. 2.2:
 //   r = sigmoid(X W^r);   r^topk, I = TopK(r, k).
 //
-// The selection is a per-row radix select on an order-preserving uint32
-// image of the fp32 scores (4 passes of 8 bits, most significant first),
-// which finds the exact k-th largest key.  With first_token, token 0 gets a
-// key above every score's (0xFFFFFFFF; a finite or infinite score maps at most
-// to 0xFF800000), so it is always kept and the other k-1 come from the rest.
-// A final in-order compaction keeps every key above the k-th largest plus the
-// lowest-index keys equal to it, so I comes out
-// ascending (the order the causal mask works in) and ties go to the lower
-// token index.  Output positions come from one block-wide prefix sum of the
-// per-segment counts, so no sort is needed.
+// The selection works on an order-preserving uint32 image of the fp32 scores
+// (topk_select_kernel); an in-order compaction keeps every key above the k-th
+// largest plus the lowest-index keys equal to it, so I comes out ascending (the
+// order the causal mask works in) and ties go to the lower token index.  Output
+// positions come from block-wide prefix sums, so no sort is needed.
 #include <algorithm>
 #include <mutex>
 
@@ -184,15 +179,284 @@ __device__ __forceinline__ uint32_t order_key(float f) {
     if (u == 0x80000000u) u = 0u;
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
-// The score an order key came from (exact, except that both zeros give +0).
-__device__ __forceinline__ float key_score(uint32_t key) {
-    return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
+constexpr int kSelThreads = 1024;
+constexpr int kSelMaxVec = 4;     // float4 per thread: rows up to 16384 scores
+constexpr int kSelCand = 64;      // candidates ranked directly
+
+// Four scores s[t .. t+3] (zeros past T).
+__device__ __forceinline__ float4 load_scores(const float *s, int t, int T, bool vec) {
+    if (vec && t + 4 <= T) return __ldg(reinterpret_cast<const float4 *>(s + t));
+    return make_float4(t < T ? __ldg(s + t) : 0.f, t + 1 < T ? __ldg(s + t + 1) : 0.f,
+                       t + 2 < T ? __ldg(s + t + 2) : 0.f, t + 3 < T ? __ldg(s + t + 3) : 0.f);
 }
 
-constexpr int kSelThreads = 1024;   // upper bound; launches use 256 or 1024
-// Rows up to this many scores keep their order keys in shared memory for all
-// five passes over them (four radix passes and the compaction).
-constexpr int kSelStagedMax = 16384;
+// One CTA per row; thread t holds the scores 4 t + 4 v blockDim .. +3, v < V, in
+// registers (V blockDim 4 >= T).  The k-th largest key is found by narrowing a key
+// range [lo, lo + NB 2^shift): a histogram of the keys inside it over NB = 2
+// blockDim equal bins, first over the row's own range [min, max], then over the
+// bin that holds the k-th key, until
+//   the bin's keys are all kept (router scores with a clear gap), or
+//   at most kSelCand keys are left: every warp ranks them directly, or
+//   the bin is one key wide: ties, kept in token order.
+// With bins over the row's range instead of fixed digits of the key (sigmoid
+// scores share two or three top bytes), one histogram is the rule; a pass costs
+// three barriers.  What bounds it is the latency of that chain, not the few KB a
+// row has.  Alone, against four 8-bit radix passes over keys in shared memory:
+// 64 x 8192 k 256 13.3 -> 9.4 us (11.1 -> 7.3 with a margin after the k-th
+// score), 1024 x 1024 k 64 12.3 -> 9.0, 1024 x 4096 k 64 29.3 -> 22.4, 32 x 4096
+// k 2048 10.1 -> 9.0, 48 x 1000 k 125 7.9 -> 5.5.
+// With first_token, token 0 is kept and k - 1 others are chosen.
+template <int V>
+__global__ void __launch_bounds__(kSelThreads)
+topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__restrict__ I,
+                   float *__restrict__ rsel, int B, int H, int32_t *__restrict__ gidx,
+                   float *__restrict__ rsel_hm, int first_token, unsigned long long *span) {
+    __shared__ uint32_t hist[2][2 * kSelThreads];
+    __shared__ uint32_t wsum[32], csum[V][32], esum[V][32];
+    __shared__ uint32_t wmin[32], wmax[32], sh_bin, sh_left, sh_in, sh_n;
+    __shared__ uint32_t cand_key[kSelCand];
+    __shared__ int cand_tok[kSelCand];
+    constexpr uint32_t kAll = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
+    const int nwarps = nthr >> 5, NB = 2 * nthr;
+    const int row = blockIdx.x;
+    const float *s = scores + (size_t)row * T;
+    const bool vec = (T & 3) == 0 && (reinterpret_cast<uintptr_t>(scores) & 15) == 0;
+    for (int i = tid; i < NB; i += nthr) hist[0][i] = 0u;
+    if (tid == 0) sh_n = 0u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // scores from the router kernel
+    span_begin(span);
+    float4 sc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) sc[v] = load_scores(s, 4 * (tid + v * nthr), T, vec);
+    uint32_t key[V][4];
+    uint32_t live = 0u;   // bit 4 v + e: a token to rank
+    uint32_t mn = 0xffffffffu, mx = 0u;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const float x[4] = {sc[v].x, sc[v].y, sc[v].z, sc[v].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int t = 4 * (tid + v * nthr) + e;
+            key[v][e] = order_key(x[e]);
+            if (t < T && !(first_token && t == 0)) {
+                live |= 1u << (4 * v + e);
+                mn = min(mn, key[v][e]);
+                mx = max(mx, key[v][e]);
+            }
+        }
+    }
+    mn = __reduce_min_sync(kAll, mn);
+    mx = __reduce_max_sync(kAll, mx);
+    if (lane == 0) {
+        wmin[warp] = mn;
+        wmax[warp] = mx;
+    }
+    __syncthreads();
+    mn = __reduce_min_sync(kAll, lane < nwarps ? wmin[lane] : 0xffffffffu);
+    mx = __reduce_max_sync(kAll, lane < nwarps ? wmax[lane] : 0u);
+    const uint32_t lg_nb = 31 - __clz(NB);   // bins used: a power of two <= NB
+    uint32_t lo = mn;
+    uint32_t remaining = (uint32_t)(first_token ? k - 1 : k);
+    // shift: the smallest with (max - lo) >> shift < 2^lg_nb
+    const uint32_t range = mx - lo;
+    const int bits = range == 0u ? 0 : 32 - __clz(range);
+    int shift = bits > (int)lg_nb ? bits - (int)lg_nb : 0;
+    uint32_t width_m1 = range;     // keys lo .. lo + width_m1 are in the range
+    // what is kept: keys above thr, and keys equal to it up to token thr_tok
+    // (or, with ties, the first `left` of them in token order)
+    uint32_t thr = 0u;
+    int thr_tok = -1;
+    bool ties = false;
+    if (remaining == 0u) thr = 0xffffffffu;   // first_token with k = 1: nothing else
+    for (int pass = 0; remaining > 0u; ++pass) {
+        uint32_t *hc = hist[pass & 1], *hn = hist[(pass + 1) & 1];
+        for (int i = tid; i < NB; i += nthr) hn[i] = 0u;   // read by no one this pass
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t off = key[v][e] - lo;   // below lo wraps past the range
+                if ((live >> (4 * v + e) & 1u) && off <= width_m1) atomicAdd(&hc[off >> shift], 1u);
+            }
+        __syncthreads();
+        // warp w sums bins NB - 64 (w + 1) .. +63 (largest keys first), then every
+        // warp finds the group that reaches the k-th key
+        const int b0 = NB - 64 * (warp + 1);
+        const uint32_t c0 = hc[b0 + 63 - 2 * lane], c1 = hc[b0 + 62 - 2 * lane];
+        const uint32_t tot = __reduce_add_sync(kAll, c0 + c1);
+        if (lane == 0) wsum[warp] = tot;
+        __syncthreads();
+        uint32_t incl = lane < nwarps ? wsum[lane] : 0u;
+        const uint32_t own = incl;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(kAll, incl, off);
+            if (lane >= off) incl += y;
+        }
+        const int g = __ffs(__ballot_sync(kAll, incl >= remaining)) - 1;
+        const uint32_t before = __shfl_sync(kAll, incl - own, g);
+        if (warp == g) {
+            uint32_t in2 = c0 + c1;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t y = __shfl_up_sync(kAll, in2, off);
+                if (lane >= off) in2 += y;
+            }
+            const int l = __ffs(__ballot_sync(kAll, before + in2 >= remaining)) - 1;
+            if (lane == l) {
+                const uint32_t b4 = before + in2 - (c0 + c1);   // keys in larger bins
+                const bool second = b4 + c0 < remaining;
+                sh_bin = (uint32_t)(b0 + (second ? 62 : 63) - 2 * lane);
+                sh_left = remaining - b4 - (second ? c0 : 0u);
+                sh_in = second ? c1 : c0;
+            }
+        }
+        __syncthreads();
+        remaining = sh_left;
+        const uint32_t in = sh_in;
+        lo += sh_bin << shift;
+        width_m1 = shift == 0 ? 0u : min((1u << shift) - 1u, 0xffffffffu - lo);
+        if (in == remaining) {   // the whole bin is kept
+            thr = lo;
+            thr_tok = T;
+            break;
+        }
+        if (in <= kSelCand) {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if ((live >> (4 * v + e) & 1u) && key[v][e] - lo <= width_m1) {
+                        const uint32_t at = atomicAdd(&sh_n, 1u);
+                        cand_key[at] = key[v][e];
+                        cand_tok[at] = 4 * (tid + v * nthr) + e;
+                    }
+            __syncthreads();
+            // rank of this lane's candidates; the one of rank remaining - 1 is the k-th
+            uint32_t rk[2] = {0u, 0u}, ck[2];
+            int ct[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int c = lane + 32 * u;
+                ck[u] = c < (int)in ? cand_key[c] : 0u;
+                ct[u] = c < (int)in ? cand_tok[c] : 0x7fffffff;
+            }
+            for (int c = 0; c < (int)in; ++c) {
+                const uint32_t ok = cand_key[c];
+                const int ot = cand_tok[c];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    rk[u] += ok > ck[u] || (ok == ck[u] && ot < ct[u]) ? 1u : 0u;
+            }
+            const bool h0 = lane < (int)in && rk[0] == remaining - 1u;
+            const bool h1 = lane + 32 < (int)in && rk[1] == remaining - 1u;
+            const int src = __ffs(__ballot_sync(kAll, h0 || h1)) - 1;
+            thr = __shfl_sync(kAll, h1 ? ck[1] : ck[0], src);
+            thr_tok = __shfl_sync(kAll, h1 ? ct[1] : ct[0], src);
+            break;
+        }
+        if (shift == 0) {   // more than kSelCand keys equal to lo, `remaining` of them kept
+            thr = lo;
+            ties = true;
+            break;
+        }
+        shift = shift > (int)lg_nb ? shift - (int)lg_nb : 0;
+    }
+    // The whole-bin stop keeps every key of the bin, above lo as well as lo itself
+    // (thr_tok = T); a threshold key keeps its tokens up to thr_tok.
+    uint32_t take = 0u, eq = 0u;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t bit = 1u << (4 * v + e);
+            const int t = 4 * (tid + v * nthr) + e;
+            if (!(live & bit)) {
+                if (first_token && t == 0) take |= bit;
+                continue;
+            }
+            if (key[v][e] > thr || (key[v][e] == thr && t <= thr_tok)) take |= bit;
+            if (key[v][e] == thr) eq |= bit;
+        }
+    if (ties) {
+        // the first `remaining` tokens whose key is thr: their order from one
+        // block-wide scan of the counts
+        uint32_t pre[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const uint32_t n = __popc(eq >> (4 * v) & 15u);
+            uint32_t in2 = n;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t y = __shfl_up_sync(kAll, in2, off);
+                if (lane >= off) in2 += y;
+            }
+            if (lane == 31) esum[v][warp] = in2;
+            pre[v] = in2 - n;
+        }
+        __syncthreads();
+        uint32_t base = 0u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const uint32_t w = lane < nwarps ? esum[v][lane] : 0u;
+            uint32_t at = base + __reduce_add_sync(kAll, lane < warp ? w : 0u) + pre[v];
+            base += __reduce_add_sync(kAll, w);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (eq >> (4 * v + e) & 1u) {
+                    if (at < remaining) take |= 1u << (4 * v + e);
+                    ++at;
+                }
+        }
+    }
+    uint32_t pre[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const uint32_t n = __popc(take >> (4 * v) & 15u);
+        uint32_t in2 = n;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(kAll, in2, off);
+            if (lane >= off) in2 += y;
+        }
+        if (lane == 31) csum[v][warp] = in2;
+        pre[v] = in2 - n;
+    }
+    __syncthreads();
+    const int hh = row % H, bb = row / H;
+    const size_t out = (size_t)row * k, out_hm = ((size_t)hh * B + bb) * k;
+    uint32_t base = 0u;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const uint32_t w = lane < nwarps ? csum[v][lane] : 0u;
+        uint32_t pos = base + __reduce_add_sync(kAll, lane < warp ? w : 0u) + pre[v];
+        base += __reduce_add_sync(kAll, w);
+        const float x[4] = {sc[v].x, sc[v].y, sc[v].z, sc[v].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (take >> (4 * v + e) & 1u) {
+                const int t = 4 * (tid + v * nthr) + e;
+                I[out + pos] = t;
+                rsel[out + pos] = x[e];
+                if (gidx != nullptr) {
+                    gidx[out_hm + pos] = bb * T + t;
+                    rsel_hm[out_hm + pos] = x[e];
+                }
+                ++pos;
+            }
+    }
+    // The next kernel launches only now: launched at this kernel's start, its
+    // CTAs (one per SM for the projections) sat on every SM this grid of B*H
+    // CTAs leaves idle, and the side stream's copies and zeroing found no SM
+    // until the attention kernel's tail (measured at B4 T4096 d1024 H16 k1024:
+    // a 13 us wait before the output product, 394 -> 381 us a step).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (span != nullptr) {
+        __syncthreads();
+        span_end(span);
+    }
+}
 
 // Block-wide exclusive prefix sum of v (thread order); `total` receives the
 // sum.  sh has 33 entries.  Two barriers.
@@ -225,16 +489,15 @@ __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long
     return sh[warp] + incl - v;
 }
 
-// One CTA per row, 256 to 1024 threads (chosen at launch).
-// Radix passes use two histograms in turn (the next one is cleared while the
+// Rows of more than 16384 scores: one CTA per row, four 8-bit radix passes over the
+// scores in memory.  The passes use two histograms in turn (the next one is cleared while the
 // current one fills), so a pass costs two barriers; the compaction gives each
 // thread a contiguous segment of the row and places its selected keys after
 // one block-wide scan of the per-segment counts.
 __global__ void __launch_bounds__(kSelThreads)
-topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__restrict__ I,
+topk_long_kernel(const float *__restrict__ scores, int T, int k, int32_t *__restrict__ I,
                    float *__restrict__ rsel, int B, int H, int32_t *__restrict__ gidx,
                    float *__restrict__ rsel_hm, int first_token, unsigned long long *span) {
-    extern __shared__ uint32_t keys_s[];   // the row's order keys when T <= kSelStagedMax
     __shared__ uint32_t hist[2][256];
     __shared__ unsigned long long sh[33];
     __shared__ uint32_t sh_prefix, sh_remaining, sh_done;
@@ -243,29 +506,12 @@ topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__re
     const int row = blockIdx.x;
     const float *s = scores + (size_t)row * T;
     const int tid = threadIdx.x;
-    const bool staged = T <= kSelStagedMax;
     for (int i = tid; i < 256; i += blockDim.x) hist[0][i] = 0u;
     // token 0's key under first_token: above every score's
     auto key_of = [&](int t) -> uint32_t {
         return (first_token && t == 0) ? 0xFFFFFFFFu : order_key(__ldg(s + t));
     };
-    if (staged) {
-        if ((T & 3) == 0 && (reinterpret_cast<uintptr_t>(s) & 15u) == 0) {
-            // four scores per 16-byte load, the loads of a thread issued together
-            const float4 *s4 = reinterpret_cast<const float4 *>(s);
-#pragma unroll 4
-            for (int q = tid; q < T / 4; q += blockDim.x) {
-                const float4 v = __ldg(s4 + q);
-                uint4 kk = make_uint4(order_key(v.x), order_key(v.y), order_key(v.z), order_key(v.w));
-                if (first_token && q == 0) kk.x = 0xFFFFFFFFu;
-                reinterpret_cast<uint4 *>(keys_s)[q] = kk;
-            }
-        } else {
-            for (int t = tid; t < T; t += blockDim.x) keys_s[t] = key_of(t);
-        }
-    }
     __syncthreads();
-    auto key_at = [&](int t) -> uint32_t { return staged ? keys_s[t] : key_of(t); };
 
     uint32_t prefix = 0u, mask = 0u, remaining = (uint32_t)k;
     for (int pass = 0; pass < 4; ++pass) {
@@ -276,7 +522,7 @@ topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__re
         // 700-800 cycles a pass whether the keys fall into three bins or 256;
         // aggregating equal bins per warp first (match.any) cost 1300-8100)
         for (int t = tid; t < T; t += blockDim.x) {
-            const uint32_t key = key_at(t);
+            const uint32_t key = key_of(t);
             if ((key & mask) == prefix) atomicAdd(&hc[(key >> shift) & 255u], 1u);
         }
         __syncthreads();
@@ -333,7 +579,7 @@ topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__re
     const int t0 = min(T, tid * per), t1 = min(T, t0 + per);
     uint32_t n_gt = 0u, n_eq = 0u;
     for (int t = t0; t < t1; ++t) {
-        const uint32_t key = key_at(t) & mask;
+        const uint32_t key = key_of(t) & mask;
         n_gt += key > thr ? 1u : 0u;
         n_eq += key == thr ? 1u : 0u;
     }
@@ -344,15 +590,11 @@ topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__re
     uint32_t pos = (uint32_t)(before >> 32) + min(eq_before, remaining);
     const int hh = row % H, bb = row / H;
     for (int t = t0; t < t1 && pos < (uint32_t)k; ++t) {
-        const uint32_t full = key_at(t), key = full & mask;
+        const uint32_t full = key_of(t), key = full & mask;
         bool take = key > thr;
         if (key == thr) take = eq_before++ < remaining;
         if (take) {
-            // the score from its staged key (no second read of the row), but
-            // from memory for token 0 under first_token and for a zero (-0 and
-            // +0 share a key)
-            const float v = (staged && !(first_token && t == 0) && full != 0x80000000u)
-                                ? key_score(full) : __ldg(s + t);
+            const float v = __ldg(s + t);
             I[(size_t)row * k + pos] = t;
             rsel[(size_t)row * k + pos] = v;
             if (gidx != nullptr) {
@@ -363,11 +605,6 @@ topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__re
             ++pos;
         }
     }
-    // The next kernel launches only now: launched at this kernel's start, its
-    // CTAs (one per SM for the projections) sat on every SM this grid of B*H
-    // CTAs leaves idle, and the side stream's copies and zeroing found no SM
-    // until the attention kernel's tail (measured at B4 T4096 d1024 H16 k1024:
-    // a 13 us wait before the output product, 394 -> 381 us a step).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (span != nullptr) {
         __syncthreads();
@@ -493,18 +730,21 @@ cudaError_t launch_select(int rows, int T, int k, const float *scores, int32_t *
                           int B, int H, int32_t *gidx, float *rsel_hm, cudaStream_t stream,
                           bool first_token) {
     if (rows <= 0) return cudaSuccess;
-    const cudaError_t attr =
-        allow_smem((const void *)topk_select_kernel, kSelStagedMax * (int)sizeof(uint32_t));
-    if (attr != cudaSuccess) return attr;
-    const size_t smem = T <= kSelStagedMax ? sizeof(uint32_t) * (size_t)T : 0;
-    // about four keys per thread, 256..1024 threads; at most 512 once rows fill
-    // the GPU (measured best at rows x T = 128 x 1024, 1024 x 1024, 32..256 x
-    // 4096, 512 and 1024 x 4096, 64 x 8192)
-    int threads = T / 4 < 256 ? 256 : (T / 4 > 1024 ? 1024 : (T / 4 + 31) / 32 * 32);
-    if (rows >= 512 && threads > 512) threads = 512;
-    cudaError_t e = launch_ahead(topk_select_kernel, dim3(rows), dim3(threads), smem, stream,
-                               scores, T, k, I, rsel, B, H, gidx, rsel_hm, first_token ? 1 : 0,
-                               active_span());
+    if (T > 16 * kSelThreads) {
+        const cudaError_t e = launch_ahead(topk_long_kernel, dim3(rows), dim3(kSelThreads), 0, stream,
+                                           scores, T, k, I, rsel, B, H, gidx, rsel_hm,
+                                           first_token ? 1 : 0, active_span());
+        note_launches(1);
+        return e;
+    }
+    // four scores per thread while all rows' threads fit the 152 SMs at once
+    // (1024 each at 64 registers) and a CTA has at most 1024; else eight or sixteen
+    int V = 1;
+    auto threads = [&]() { return ((T + 4 * V - 1) / (4 * V) + 31) / 32 * 32; };
+    while (V < kSelMaxVec && (threads() > kSelThreads || (long long)rows * threads() > 152 * 1024)) V *= 2;
+    auto kern = V == 1 ? topk_select_kernel<1> : V == 2 ? topk_select_kernel<2> : topk_select_kernel<4>;
+    const cudaError_t e = launch_ahead(kern, dim3(rows), dim3(threads()), 0, stream, scores, T, k, I,
+                                       rsel, B, H, gidx, rsel_hm, first_token ? 1 : 0, active_span());
     note_launches(1);
     return e;
 }

@@ -72,6 +72,32 @@ def test_topk_bit_exact(kind, T, k):
         np.testing.assert_array_equal(rs[r].view(np.uint32), s[r][Iref].view(np.uint32))
 
 
+# rows held in registers, four, eight or sixteen scores per thread (by length and
+# by number of rows), their longest (16384) and the shortest beyond; outliers that
+# leave every other score in one bin of the first histogram, with and without ties
+@pytest.mark.parametrize("kind", ["uniform", "ties", "outliers", "outliers_ties"])
+@pytest.mark.parametrize("rows,T,k", [(2, 33, 33), (3, 8193, 70), (2, 16381, 16000),
+                                      (2, 16384, 65), (2, 16385, 65), (1300, 130, 17),
+                                      (700, 1030, 200)])
+def test_topk_row_shapes_bit_exact(kind, rows, T, k):
+    rng = np.random.default_rng(T * 17 + rows)
+    if kind.startswith("outliers"):
+        s = 0.5 + 1e-7 * rng.integers(0, 4 if kind == "outliers_ties" else T, size=(rows, T))
+        s = s.astype(np.float32)
+        s[:, 1] = np.float32(3e38)
+        s[:, 5] = -np.inf
+        s[:, 9] = np.inf
+    else:
+        s = score_rows(kind, rows, T, rng, k)
+    I, rs = mosa.mosa_topk(torch.from_numpy(s).cuda(), k)
+    I, rs = I.cpu().numpy(), rs.cpu().numpy()
+    order = np.argsort(-s.astype(np.float64), axis=1, kind="stable")[:, :k]
+    ref = np.sort(order, axis=1)
+    np.testing.assert_array_equal(I, ref)
+    np.testing.assert_array_equal(rs.view(np.uint32),
+                                  np.take_along_axis(s, ref, axis=1).view(np.uint32))
+
+
 # ---------------------------------------------------- small full parity ----
 
 SMALL = [
