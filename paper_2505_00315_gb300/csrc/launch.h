@@ -82,9 +82,10 @@ cudaError_t launch_rope(void *p0, int col0_0, void *p1, int col0_1, bool pair, i
                         long long rows, const int32_t *gidx, const RopeTable &tab, float dir,
                         cudaStream_t s);
 
-// F1, Sec. 2.2 router: r_full[b,h,t] = sigmoid(X[b,t,:] . W_r[:,h]) in fp32.
+// F1, Sec. 2.2 router: r_full[b,h,t] = sigmoid(X[b,t,:] . W_r[:,h]) in fp32, on CUDA
+// cores; zeroes *status (not null) first.
 cudaError_t launch_router(const Dims &dm, const void *X, const void *Wr, float *r_full,
-                          cudaStream_t stream);
+                          uint32_t *status, cudaStream_t stream);
 // F1 choosing the tensor-core kernel where it applies.  wr_pad (optional):
 // room for a [d, H rounded up to 64] bf16 copy of W_r, used by the
 // tensor-core router when H % 64 != 0; zero_status: zero the status word

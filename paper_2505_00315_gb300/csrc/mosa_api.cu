@@ -363,10 +363,9 @@ mosa_status forward_routed(const Dims &dm, const void *X, const void *W_r, const
         return forward_tc(dm, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf, true, nullptr, nullptr,
                           sv, s, *res);
     MOSA_TRY(begin_timeline_call(kForwardStages, s));
-    MOSA_TRY(cudaMemsetAsync(sv.status, 0, sizeof(uint32_t), s));
     {
         StageScope st_(kStageRouter, s);
-        MOSA_TRY(launch_router_auto(dm, X, W_r, rf, sv.status, s));
+        MOSA_TRY(launch_router_auto(dm, X, W_r, rf, sv.status, s, nullptr, /*zero_status=*/true));
     }
     {
         StageScope st_(kStageSelect, s);

@@ -80,7 +80,8 @@ __device__ __forceinline__ void widen8(const bf16 *p, float (&v)[8]) {
 template <class E, int HT>
 __global__ void __launch_bounds__(RouterTile<HT>::THREADS)
     router_rows_kernel(const E *__restrict__ X, const E *__restrict__ Wr, float *__restrict__ r_full,
-                       int M, int T, int H, int d) {
+                       int M, int T, int H, int d, uint32_t *status) {
+    if (status != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = 0u;
     constexpr int THREADS = RouterTile<HT>::THREADS, TOK = RouterTile<HT>::TOK;
     constexpr int KC = RouterTile<HT>::KC;
     constexpr int TM = HT / 16;                    // tokens per thread
@@ -651,7 +652,7 @@ __global__ void dense_rows_kernel(long long n, long long rows_per_head,
 
 template <class E, int HT>
 static cudaError_t router_rows(const Dims &dm, const void *X, const void *Wr, float *r_full,
-                               cudaStream_t stream) {
+                               uint32_t *status, cudaStream_t stream) {
     const int M = dm.B * dm.T;
     constexpr int tok = RouterTile<HT>::TOK;
     const dim3 grid((M + tok - 1) / tok, (dm.H + HT - 1) / HT);
@@ -659,27 +660,31 @@ static cudaError_t router_rows(const Dims &dm, const void *X, const void *Wr, fl
     const cudaError_t e = allow_smem((const void *)router_rows_kernel<E, HT>, smem);
     if (e != cudaSuccess) return e;
     router_rows_kernel<E, HT><<<grid, RouterTile<HT>::THREADS, smem, stream>>>(
-        (const E *)X, (const E *)Wr, r_full, M, dm.T, dm.H, dm.d);
+        (const E *)X, (const E *)Wr, r_full, M, dm.T, dm.H, dm.d, status);
     note_launches(1);
     return cudaGetLastError();
 }
 
 template <class E>
 static cudaError_t router_t(const Dims &dm, const void *X, const void *Wr, float *r_full,
-                            cudaStream_t stream) {
+                            uint32_t *status, cudaStream_t stream) {
     if ((reinterpret_cast<uintptr_t>(X) & 15) != 0) {   // no 16-byte loads of its rows
+        if (status != nullptr) {
+            const cudaError_t e = cudaMemsetAsync(status, 0, sizeof(uint32_t), stream);
+            if (e != cudaSuccess) return e;
+        }
         RouterOp<E> op{dm.B * dm.T, dm.H, dm.d, dm.T, dm.H, (const E *)X, (const E *)Wr, r_full};
         return launch_simt_gemm(op, 1, stream);
     }
-    if (dm.H <= 16) return router_rows<E, 16>(dm, X, Wr, r_full, stream);
-    if (dm.H <= 32) return router_rows<E, 32>(dm, X, Wr, r_full, stream);
-    return router_rows<E, 64>(dm, X, Wr, r_full, stream);
+    if (dm.H <= 16) return router_rows<E, 16>(dm, X, Wr, r_full, status, stream);
+    if (dm.H <= 32) return router_rows<E, 32>(dm, X, Wr, r_full, status, stream);
+    return router_rows<E, 64>(dm, X, Wr, r_full, status, stream);
 }
 
 cudaError_t launch_router(const Dims &dm, const void *X, const void *Wr, float *r_full,
-                          cudaStream_t stream) {
-    return dm.bf16 ? router_t<bf16>(dm, X, Wr, r_full, stream)
-                   : router_t<float>(dm, X, Wr, r_full, stream);
+                          uint32_t *status, cudaStream_t stream) {
+    return dm.bf16 ? router_t<bf16>(dm, X, Wr, r_full, status, stream)
+                   : router_t<float>(dm, X, Wr, r_full, status, stream);
 }
 
 // W_r [d,H] -> Wp [d,Hp], columns H..Hp-1 zero, and the status word zeroed
@@ -718,12 +723,14 @@ cudaError_t launch_router_auto(const Dims &dm, const void *X, const void *Wr, fl
                                                  zero_status ? status : nullptr);
         note_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else if (zero_status) {
+    } else if (tc && zero_status) {
         if ((e = cudaMemsetAsync(status, 0, sizeof(uint32_t), stream)) != cudaSuccess) return e;
     }
     if (tc && tc_router(dm, X, pad ? wr_pad : Wr, pad ? hp64 : dm.H, r_full, status, stream, &e))
         return e;
-    return launch_router(dm, X, Wr, r_full, stream);
+    // (launched without the early-launch attribute, so the status word is zeroed
+    // after all earlier work on the stream)
+    return launch_router(dm, X, Wr, r_full, zero_status ? status : nullptr, stream);
 }
 
 cudaError_t launch_select(int rows, int T, int k, const float *scores, int32_t *I, float *rsel,
