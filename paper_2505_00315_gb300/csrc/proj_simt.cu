@@ -261,11 +261,12 @@ struct WBwdOp {
 
 // One warp per selected row: dr = <A, G>, dA = r G (rounded to storage),
 // D = rowsum(dA o A), dlogit = dr r (1 - r).
+// (Pointers without __restrict__: see attn_fwd_simt_kernel.)
 template <class TS>
-__global__ void out_bwd_rows_kernel(const float *__restrict__ G, const float *__restrict__ A,
-                                    const float *__restrict__ rsel, void *__restrict__ dA,
-                                    float *__restrict__ Dd, float *__restrict__ dlogit,
-                                    void *__restrict__ dQKV, long long rows, int hp) {
+__global__ void out_bwd_rows_kernel(const float *G, const float *A,
+                                    const float *rsel, void *dA,
+                                    float *Dd, float *dlogit,
+                                    void *dQKV, long long rows, int hp) {
     tc::pdl_wait();
     const long long row = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;

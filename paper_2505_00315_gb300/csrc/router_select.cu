@@ -184,11 +184,12 @@ constexpr int kSelThreads = 1024;
 constexpr int kSelMaxVec = 4;     // float4 per thread: rows up to 16384 scores
 constexpr int kSelCand = 64;      // candidates ranked directly
 
-// Four scores s[t .. t+3] (zeros past T).
+// Four scores s[t .. t+3] (zeros past T).  Plain loads, not __ldg, which the compiler
+// may move ahead of the wait for the kernel that writes the scores.
 __device__ __forceinline__ float4 load_scores(const float *s, int t, int T, bool vec) {
-    if (vec && t + 4 <= T) return __ldg(reinterpret_cast<const float4 *>(s + t));
-    return make_float4(t < T ? __ldg(s + t) : 0.f, t + 1 < T ? __ldg(s + t + 1) : 0.f,
-                       t + 2 < T ? __ldg(s + t + 2) : 0.f, t + 3 < T ? __ldg(s + t + 3) : 0.f);
+    if (vec && t + 4 <= T) return *reinterpret_cast<const float4 *>(s + t);
+    return make_float4(t < T ? s[t] : 0.f, t + 1 < T ? s[t + 1] : 0.f, t + 2 < T ? s[t + 2] : 0.f,
+                       t + 3 < T ? s[t + 3] : 0.f);
 }
 
 // One CTA per row; thread t holds the scores 4 t + 4 v blockDim .. +3, v < V, in
@@ -209,9 +210,8 @@ __device__ __forceinline__ float4 load_scores(const float *s, int t, int T, bool
 // With first_token, token 0 is kept and k - 1 others are chosen.
 template <int V>
 __global__ void __launch_bounds__(kSelThreads)
-topk_select_kernel(const float *__restrict__ scores, int T, int k, int32_t *__restrict__ I,
-                   float *__restrict__ rsel, int B, int H, int32_t *__restrict__ gidx,
-                   float *__restrict__ rsel_hm, int first_token, unsigned long long *span) {
+topk_select_kernel(const float *scores, int T, int k, int32_t *I, float *rsel, int B, int H,
+                   int32_t *gidx, float *rsel_hm, int first_token, unsigned long long *span) {
     __shared__ uint32_t hist[2][2 * kSelThreads];
     __shared__ uint32_t wsum[32], csum[V][32], esum[V][32];
     __shared__ uint32_t wmin[32], wmax[32], sh_bin, sh_left, sh_in, sh_n;
@@ -496,9 +496,9 @@ __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long
 // thread a contiguous segment of the row and places its selected keys after
 // one block-wide scan of the per-segment counts.
 __global__ void __launch_bounds__(kSelThreads)
-topk_long_kernel(const float *__restrict__ scores, int T, int k, int32_t *__restrict__ I,
-                   float *__restrict__ rsel, int B, int H, int32_t *__restrict__ gidx,
-                   float *__restrict__ rsel_hm, int first_token, unsigned long long *span) {
+topk_long_kernel(const float *scores, int T, int k, int32_t *I,
+                   float *rsel, int B, int H, int32_t *gidx,
+                   float *rsel_hm, int first_token, unsigned long long *span) {
     __shared__ uint32_t hist[2][256];
     __shared__ unsigned long long sh[33];
     __shared__ uint32_t sh_prefix, sh_remaining, sh_done;
@@ -510,7 +510,7 @@ topk_long_kernel(const float *__restrict__ scores, int T, int k, int32_t *__rest
     for (int i = tid; i < 256; i += blockDim.x) hist[0][i] = 0u;
     // token 0's key under first_token: above every score's
     auto key_of = [&](int t) -> uint32_t {
-        return (first_token && t == 0) ? 0xFFFFFFFFu : order_key(__ldg(s + t));
+        return (first_token && t == 0) ? 0xFFFFFFFFu : order_key(s[t]);
     };
     __syncthreads();
 
@@ -595,7 +595,7 @@ topk_long_kernel(const float *__restrict__ scores, int T, int k, int32_t *__rest
         bool take = key > thr;
         if (key == thr) take = eq_before++ < remaining;
         if (take) {
-            const float v = __ldg(s + t);
+            const float v = s[t];
             I[(size_t)row * k + pos] = t;
             rsel[(size_t)row * k + pos] = v;
             if (gidx != nullptr) {
