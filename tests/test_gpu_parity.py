@@ -168,6 +168,48 @@ def test_small_forward_backward_full_parity(cfg, kernel_path):
         assert_close(name, g[gname], ref[name], cfg.dtype)
 
 
+# Products through bf16 planes (fp32 storage; bf16 with a head size other than 64) with
+# more than 152 tiles, so that CTAs walk over several, and edges in every
+# dimension: rows and columns past a tile, a K block of 8, reduction splits
+@pytest.mark.parametrize("cfg", [
+    W.MosaConfig("planes_f32", B=2, T=200, d=520, H=26, hp=64, k=77, dtype="f32", seed=71),
+    W.MosaConfig("planes_f32_splits", B=3, T=700, d=72, H=2, hp=32, k=345, dtype="f32", seed=72),
+    W.MosaConfig("planes_hp128", B=2, T=200, d=392, H=22, hp=128, k=66, dtype="bf16", seed=73),
+    W.MosaConfig("planes_hp16", B=3, T=150, d=264, H=33, hp=16, k=50, dtype="bf16", seed=74),
+], ids=lambda c: c.name)
+def test_plane_products_many_tiles_parity(cfg):
+    x = W.make_inputs(cfg)
+    Y, I, _, _ = oracle.forward(x["X"], *weights(x), k=cfg.k)
+    g = run_layer(cfg, x, backward=True)
+    np.testing.assert_array_equal(g["I"], I)
+    assert_close("Y", g["Y"], Y, cfg.dtype)
+    ref = oracle.backward(x["X"], *weights(x), I=I, dY=x["dY"])
+    for name in ("dX", "dWr", "dWq", "dWk", "dWv", "dWo"):
+        gname = name[:2] + "_" + name[2:].lower() if name != "dX" else "dX"
+        assert_close(name, g[gname], ref[name], cfg.dtype)
+
+
+def test_non_finite_f32_inputs_as_on_cuda_cores(monkeypatch):
+    # An infinity cut into planes is NaN in the plane products; the results around
+    # it must be those of plain multiply-adds: infinite or NaN in the same places
+    # and unchanged everywhere else.
+    cfg = W.MosaConfig("nonfinite_f32", B=2, T=120, d=72, H=3, hp=32, k=40, dtype="f32", seed=75)
+    x = W.make_inputs(cfg)
+    x["X"][0, 7, 3] = np.inf
+    x["X"][1, 5, 9] = np.nan
+    x["Wo"][1, 4, 11] = -np.inf
+    x["dY"][0, 30, 2] = np.inf
+    a = run_layer(cfg, x, backward=True)
+    monkeypatch.setenv("MOSA_FORCE_SIMT", "1")
+    b = run_layer(cfg, x, backward=True)
+    np.testing.assert_array_equal(a["I"], b["I"])
+    for n in ("Y", "dX", "dW_r", "dW_q", "dW_k", "dW_v", "dW_o"):
+        fin = np.isfinite(b[n])
+        np.testing.assert_array_equal(np.isfinite(a[n]), fin, err_msg=n)
+        np.testing.assert_array_equal(a[n][~fin], b[n][~fin], err_msg=n)   # NaN equal to NaN
+        np.testing.assert_allclose(a[n][fin], b[n][fin], rtol=1e-4, atol=1e-4, err_msg=n)
+
+
 # ------------------------------------ first token always kept (Sec. 3.2) ----
 
 FIRST = [
