@@ -27,6 +27,7 @@
 // Warps: 0 TMA producer, 1 MMA issuer, 2 TMEM owner, 3 TMA stores; 4-11 gather,
 // softmax and epilogues, two per TMEM lane quadrant (warp w serves tile rows
 // 32 (w % 4) .. +31 and column half (w - 4) / 4).  Every wait is bounded.
+#include <algorithm>
 #include <mutex>
 
 #include "launch.h"
@@ -103,7 +104,11 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b0 = blockIdx.x * p.U, h = blockIdx.y;
     const int nkb = (p.d + 63) / 64;
-    const int nch = (p.d + kChunk - 1) / kChunk;
+    // this CTA's output chunks: all of them, or its share (gridDim.z CTAs per tile)
+    const int all_ch = (p.d + kChunk - 1) / kChunk;
+    const int ch0 = (int)blockIdx.z * all_ch / (int)gridDim.z;
+    const int nch = ((int)blockIdx.z + 1) * all_ch / (int)gridDim.z - ch0;
+    const bool saves = blockIdx.z == 0;   // writes what the backward reads
     const size_t row_base = (size_t)h * p.Mtok + (size_t)b0 * p.k;  // head row of tile row 0
     // P pair tile [half][key block] over the start of the ring
     uint8_t(*ptile)[2][kHalf] = reinterpret_cast<uint8_t(*)[2][kHalf]>(&sm.ring[0][0]);
@@ -177,7 +182,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
                     uint8_t *dst = buf ? &sm.v[0][0] : &sm.k[0][0];
                     mbar_expect_tx(fb, 4 * 8192);
                     for (int j = 0; j < 4; ++j)
-                        tma_load_3d(smem_u32(dst + j * 8192), &p.mWo, fb, c * kChunk + 64 * j, 0, h);
+                        tma_load_3d(smem_u32(dst + j * 8192), &p.mWo, fb, (ch0 + c) * kChunk + 64 * j, 0, h);
                     nc = c + 1;
                 }
             }
@@ -270,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
         // ------------------------------------------------- TMA stores
         if (lane == 0) {
             // Q, K, V pairs straight from the attention operand tiles
-            bool ok = wait_or_abort(sm, sm.qkv_staged, 0, p.status);
+            bool ok = wait_or_abort(sm, sm.qkv_staged, 0, p.status) && saves;
             if (ok) {
                 uint8_t(*tiles[3])[kHalf] = {sm.q, sm.k, sm.v};
                 for (int j = 0; j < 3; ++j)
@@ -397,7 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
         mbar_arrive(smem_u32(&sm.ar_ready));
         const bool live = __all_sync(0xffffffffu, ok && !*(volatile int *)&sm.abort);
         uint8_t *xb = stage_area + (warp - 4) * 4096;
-        if (live && ch == 0 && valid) p.lse[grow0 + lane] = (m + log2f(l)) * 0.69314718055994531f;
+        if (live && saves && ch == 0 && valid) p.lse[grow0 + lane] = (m + log2f(l)) * 0.69314718055994531f;
 
         // ------------------------------------- phase 4: scatter-add into Y
         const int cu = lane & 7;
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fwd_kernel(const __grid_con
                 float v[32];
                 tmem_ld32(tb + s0, v);
                 stage_f32x32(xb, v, 1.f, lane);
-                const int n = c * kChunk + s0 + 4 * cu;
+                const int n = (ch0 + c) * kChunk + s0 + 4 * cu;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int rl = (lane >> 3) + 4 * i;
@@ -481,7 +486,13 @@ cudaError_t tc_fused_forward(const Dims &dm, const void *X, const void *Wq, cons
     p.span = active_span();
     const cudaError_t attr = allow_smem((const void *)fused_fwd_kernel, kSmem);
     if (attr != cudaSuccess) return attr;
-    const dim3 grid((dm.B + p.U - 1) / p.U, dm.H);
+    // Few tiles: the output chunks of a tile (about 3 us each) go to several CTAs, each
+    // of which computes the tile's attention for itself on an SM that would idle
+    // (B1 T1531 d768 H12 k95, 12 tiles of 3 chunks: 20 -> 15 us).  From 77
+    // tiles on the 152 SMs have no room for a second CTA per tile.
+    const int tiles = (dm.B + p.U - 1) / p.U * dm.H;
+    const int parts = std::max(1, std::min((dm.d + kChunk - 1) / kChunk, 152 / tiles));
+    const dim3 grid((dm.B + p.U - 1) / p.U, dm.H, parts);
     cudaError_t e = launch_ahead(fused_fwd_kernel, grid, dim3(kThreads), kSmem, s, p);
     note_launches(1);
     return e;

@@ -189,6 +189,24 @@ def test_plane_products_many_tiles_parity(cfg):
         assert_close(name, g[gname], ref[name], cfg.dtype)
 
 
+# Fused forward with few tiles: a tile's output columns shared by several CTAs, with
+# a last column block cut short and one block more than CTAs
+@pytest.mark.parametrize("cfg", [
+    W.MosaConfig("few_tiles", B=3, T=150, d=600, H=2, hp=64, k=50, dtype="bf16", seed=76),
+    W.MosaConfig("few_tiles_uneven", B=6, T=140, d=1288, H=8, hp=64, k=128, dtype="bf16", seed=77),
+], ids=lambda c: c.name)
+def test_fused_forward_few_tiles_parity(cfg):
+    x = W.make_inputs(cfg)
+    Y, I, _, _ = oracle.forward(x["X"], *weights(x), k=cfg.k)
+    g = run_layer(cfg, x, backward=True)
+    np.testing.assert_array_equal(g["I"], I)
+    assert_close("Y", g["Y"], Y, cfg.dtype)
+    ref = oracle.backward(x["X"], *weights(x), I=I, dY=x["dY"])
+    for name in ("dX", "dWq", "dWo"):
+        gname = name[:2] + "_" + name[2:].lower() if name != "dX" else "dX"
+        assert_close(name, g[gname], ref[name], cfg.dtype)
+
+
 def test_non_finite_f32_inputs_as_on_cuda_cores(monkeypatch):
     # An infinity cut into planes is NaN in the plane products; the results around
     # it must be those of plain multiply-adds: infinite or NaN in the same places
