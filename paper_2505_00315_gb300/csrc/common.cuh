@@ -158,6 +158,8 @@ struct Dims {
     bool first_token;   // token 0 always kept, k-1 more by score (Sec. 3.2)
     bool rope;          // rotary position encoding of Q and K (Sec. 2.2)
     bool accumulate;    // Y (forward) and dX (backward) are added into, not overwritten
+    bool keep_status = false;   // the caller has zeroed the status word
+    bool shared_x16 = false;    // another head group's call makes the fp16 copy of X
     long long rows() const { return (long long)H * B * k; }
     size_t esize() const { return bf16 ? 2 : 4; }
 };

@@ -116,10 +116,22 @@ constexpr uint32_t kBackwardStages = (1u << kStageOutBwd) | (1u << kStageAttnBwd
 //   backward: dW_o, the W_r transpose and (except on the fp16 path, where
 //             the attention backward does it) the zeroing of dX run beside
 //             G -> attention backward; then dX and dW run side by side.
-// A hybrid call runs the MoSA heads and then the dense heads, each this way.
+// A hybrid call runs the MoSA heads and the dense heads each this way, side by
+// side where both are on the tensor cores: the dense heads on streams of their own, up to
+// their output product (dX product in the backward), which adds into what the
+// MoSA heads wrote and waits for them.
 struct DevResources {
     cudaStream_t side = nullptr;
     cudaEvent_t ev[4] = {};
+    // hybrid calls: the dense heads' own pair of streams
+    cudaStream_t dense = nullptr, dense_side = nullptr;
+    cudaEvent_t dense_ev[4] = {}, fork = nullptr, heads_done = nullptr, dense_done = nullptr;
+    DevResources dense_set() const {
+        DevResources d;
+        d.side = dense_side;
+        for (int i = 0; i < 4; ++i) d.ev[i] = dense_ev[i];
+        return d;
+    }
 };
 constexpr int kMaxDev = 64;
 constexpr int kMaxPrio = 8;   // stream priorities 0, -1, ..
@@ -141,12 +153,16 @@ DevResources *dev_resources(int prio) {
     std::lock_guard<std::mutex> lk(g_res_mu);
     DevResources &r = g_res[dev][prio];
     if (r.side == nullptr) {
-        if (cudaStreamCreateWithPriority(&r.side, cudaStreamNonBlocking, -prio) != cudaSuccess) {
-            r.side = nullptr;
-            return nullptr;
+        for (cudaStream_t *st : {&r.dense, &r.dense_side, &r.side})
+            if (cudaStreamCreateWithPriority(st, cudaStreamNonBlocking, -prio) != cudaSuccess) {
+                r.side = nullptr;
+                return nullptr;
+            }
+        for (int i = 0; i < 11; ++i) {
+            cudaEvent_t *e = i < 4 ? &r.ev[i] : i < 8 ? &r.dense_ev[i - 4]
+                             : i == 8 ? &r.fork : i == 9 ? &r.heads_done : &r.dense_done;
+            if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
         }
-        for (auto &e : r.ev)
-            if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     }
     return &r;
 }
@@ -198,14 +214,16 @@ mosa_status forward_heads(const Dims &dm, const void *X, const void *W_q, const 
 mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const void *W_q,
                        const void *W_k, const void *W_v, const void *W_o, float *Y, int32_t *I,
                        float *r_sel, float *rf, bool route, const int32_t *I_in,
-                       const float *rsel_in, const Saved &sv, cudaStream_t s, DevResources &r) {
+                       const float *rsel_in, const Saved &sv, cudaStream_t s, DevResources &r,
+                       cudaEvent_t before_out = nullptr) {
     set_span_base(sv.spans);   // measurement: this call's kernel-span slots
     MOSA_TRY(begin_timeline_call(kForwardStages, s));
     const size_t ny = (size_t)dm.B * dm.T * dm.d;
     // A call that adds into Y continues the status word of the call that wrote it.
     if (route) {
         StageScope st_(kStageRouter, s);
-        MOSA_TRY(launch_router_auto(dm, X, W_r, rf, sv.status, s, sv.Wr64, !dm.accumulate));
+        MOSA_TRY(launch_router_auto(dm, X, W_r, rf, sv.status, s, sv.Wr64,
+                                    !dm.accumulate && !dm.keep_status));
     } else if (!dm.accumulate) {
         MOSA_TRY(cudaMemsetAsync(sv.status, 0, sizeof(uint32_t), s));
     }
@@ -221,7 +239,8 @@ mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const voi
     // made here beside TopK, whose grid (one CTA per (b, h) row) leaves most
     // SMs idle
     if (dqkv_f16(dm))
-        MOSA_TRY(tc_f16_copies(dm, X, W_q, W_k, W_v, attn_f16(dm) ? W_o : nullptr, sv, r.side));
+        MOSA_TRY(tc_f16_copies(dm, dm.shared_x16 ? nullptr : X, W_q, W_k, W_v,
+                               attn_f16(dm) ? W_o : nullptr, sv, r.side));
     if (route) {
         StageScope st_(kStageSelect, s);
         MOSA_TRY(launch_select(dm.B * dm.H, dm.T, dm.k, rf, I, r_sel, dm.B, dm.H, sv.gidx,
@@ -240,6 +259,7 @@ mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const voi
     }
     if (fused) {
         MOSA_TRY(cudaStreamWaitEvent(s, r.ev[1], 0));  // Y zeroed
+        if (before_out != nullptr) MOSA_TRY(cudaStreamWaitEvent(s, before_out, 0));
         {
             StageScope st_(kStageFwdUnit, s);
             MOSA_TRY(tc_fused_forward(dm, X, W_q, W_k, W_v, W_o, sv, Y, s));
@@ -258,6 +278,7 @@ mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const voi
         MOSA_TRY(launch_attn_fwd(dm, sv, s));
     }
     MOSA_TRY(link(r.side, s, r.ev[1]));  // Y zeroed, or the row map built
+    if (before_out != nullptr) MOSA_TRY(cudaStreamWaitEvent(s, before_out, 0));
     {
         StageScope st_(kStageOut, s);
         MOSA_TRY(tc_out(dm, W_o, sv, Y, s, false, headsum));
@@ -273,7 +294,8 @@ mosa_status forward_tc(const Dims &dm, const void *X, const void *W_r, const voi
 mosa_status backward_tc(const Dims &dm, const void *X, const void *W_r, const void *W_q,
                         const void *W_k, const void *W_v, const void *W_o, const void *dY,
                         float *dX, float *dW_r, float *dW_q, float *dW_k, float *dW_v,
-                        float *dW_o, const Saved &sv, cudaStream_t s, DevResources &r) {
+                        float *dW_o, const Saved &sv, cudaStream_t s, DevResources &r,
+                        cudaEvent_t before_dx = nullptr) {
     set_span_base(sv.spans);   // measurement: this call's kernel-span slots
     MOSA_TRY(begin_timeline_call(kBackwardStages, s));   // before the side stream forks
     cudaStream_t t = r.side;
@@ -300,6 +322,7 @@ mosa_status backward_tc(const Dims &dm, const void *X, const void *W_r, const vo
             MOSA_TRY(tc_w_bwd(dm, X, sv, dW_q, dW_k, dW_v, dW_r, t));
         }
         MOSA_TRY(cudaStreamWaitEvent(s, r.ev[1], 0));
+        if (before_dx != nullptr) MOSA_TRY(cudaStreamWaitEvent(s, before_dx, 0));
         {
             StageScope st_(kStageInBwd, s);
             MOSA_TRY(tc_in_bwd(dm, W_q, W_k, W_v, W_r, sv, dX, s, false));
@@ -342,6 +365,7 @@ mosa_status backward_tc(const Dims &dm, const void *X, const void *W_r, const vo
         MOSA_TRY(tc_w_bwd(dm, X, sv, dW_q, dW_k, dW_v, dW_r, t));
     }
     MOSA_TRY(cudaStreamWaitEvent(s, r.ev[1], 0));  // W_r transposed (and dX zeroed on the side)
+    if (before_dx != nullptr) MOSA_TRY(cudaStreamWaitEvent(s, before_dx, 0));
     {
         StageScope st_(kStageInBwd, s);
         MOSA_TRY(tc_in_bwd(dm, W_q, W_k, W_v, W_r, sv, dX, s, false, /*pos_ready=*/true));
@@ -506,6 +530,18 @@ mosa_status check_hybrid_workspace(const Hybrid &h, void *ws, size_t bytes, Hybr
     if (bytes < carve_hybrid(h, nullptr, nullptr)) return MOSA_ERR_WORKSPACE;
     carve_hybrid(h, (char *)ws, sp);
     return MOSA_OK;
+}
+
+// True when both head groups run on the tensor cores, side by side: the status
+// word is then zeroed before the fork, and one fp16 copy of X serves both.
+bool side_by_side(Hybrid *h, HybridSpace *sp) {
+    if (!h->has_dense || !use_tc(h->sparse) || !use_tc(h->dense)) return false;
+    h->sparse.keep_status = true;
+    if (dqkv_f16(h->sparse) && dqkv_f16(h->dense)) {
+        h->dense.shared_x16 = true;
+        sp->dense.X16 = sp->sparse.X16;
+    }
+    return true;
 }
 
 // ---------------------------------------------------------- graph cache
@@ -737,13 +773,27 @@ mosa_status mosa_hybrid_forward(const mosa_hybrid_shape *shape, const void *X, c
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sp.sparse.r_full;
     const int prio = priority_index((cudaStream_t)stream);
-    DevResources *rs = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
-    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources(prio) : nullptr;
+    DevResources *res = dev_resources(prio);
+    if (res == nullptr) return MOSA_ERR_CUDA;
+    const bool both = side_by_side(&h, &sp);
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
+        if (both) MOSA_TRY(cudaMemsetAsync(sp.sparse.status, 0, sizeof(uint32_t), s));
+        if (both) MOSA_TRY(cudaEventRecord(res->fork, s));
         mosa_status e = forward_routed(h.sparse, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf,
-                                       sp.sparse, s, rs);
+                                       sp.sparse, s, use_tc(h.sparse) ? res : nullptr);
         if (e != MOSA_OK || !h.has_dense) return e;
-        return forward_given(h.dense, X, D_q, D_k, D_v, D_o, nullptr, nullptr, Y, sp.dense, s, rd);
+        if (!both)
+            return forward_given(h.dense, X, D_q, D_k, D_v, D_o, nullptr, nullptr, Y, sp.dense, s,
+                                 use_tc(h.dense) ? res : nullptr);
+        MOSA_TRY(cudaEventRecord(res->heads_done, s));
+        MOSA_TRY(cudaStreamWaitEvent(res->dense, res->fork, 0));
+        DevResources d = res->dense_set();
+        set_span_base(sp.dense.spans);
+        e = forward_tc(h.dense, X, nullptr, D_q, D_k, D_v, D_o, Y, nullptr, nullptr, nullptr, false,
+                       nullptr, nullptr, sp.dense, res->dense, d, res->heads_done);
+        if (e != MOSA_OK) return e;
+        MOSA_TRY(link(res->dense, s, res->dense_done));
+        return MOSA_OK;
     };
     const GraphKey key = make_key(3, prio, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, Y, I, r_sel,
@@ -771,15 +821,30 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     const int prio = priority_index((cudaStream_t)stream);
-    DevResources *rs = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
-    DevResources *rd = h.has_dense && use_tc(h.dense) ? dev_resources(prio) : nullptr;
+    DevResources *res = dev_resources(prio);
+    if (res == nullptr) return MOSA_ERR_CUDA;
+    const bool both = side_by_side(&h, &sp);
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
+        if (both) MOSA_TRY(cudaEventRecord(res->fork, s));
         mosa_status e = backward_all(h.sparse, X, W_r, W_q, W_k, W_v, W_o, dY, dX, dW_r, dW_q,
-                                     dW_k, dW_v, dW_o, sp.sparse, s, rs);
+                                     dW_k, dW_v, dW_o, sp.sparse, s,
+                                     use_tc(h.sparse) ? res : nullptr);
         if (e != MOSA_OK || !h.has_dense) return e;
-        MOSA_TRY(cudaMemsetAsync(sp.zero_wr, 0, sp.zero_wr_bytes, s));
-        return backward_all(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q,
-                            dD_k, dD_v, dD_o, sp.dense, s, rd);
+        cudaStream_t ds = both ? res->dense : s;
+        if (both) {
+            MOSA_TRY(cudaEventRecord(res->heads_done, s));
+            MOSA_TRY(cudaStreamWaitEvent(ds, res->fork, 0));
+        }
+        MOSA_TRY(cudaMemsetAsync(sp.zero_wr, 0, sp.zero_wr_bytes, ds));
+        if (!both)
+            return backward_all(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q,
+                                dD_k, dD_v, dD_o, sp.dense, s, use_tc(h.dense) ? res : nullptr);
+        DevResources d = res->dense_set();
+        e = backward_tc(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q, dD_k, dD_v,
+                        dD_o, sp.dense, ds, d, res->heads_done);
+        if (e != MOSA_OK) return e;
+        MOSA_TRY(link(ds, s, res->dense_done));
+        return MOSA_OK;
     };
     const GraphKey key = make_key(4, prio, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, I, r_sel, dY,
