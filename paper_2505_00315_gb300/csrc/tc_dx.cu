@@ -19,6 +19,14 @@
 // product with a pair operand is two MMAs (hi, lo); on the fp16 attention
 // path (k > 128) dX reads dQ|dK|dV as single fp16 values and fp16 copies of
 // W_q|W_k|W_v, and Y reads AR as fp16 with an fp16 copy of W_o: one MMA.
+// dX with fp16 rows keeps a chunk's weight blocks instead and walks over the tiles
+// (units head, chunk, tile; kWS): a unit then loads its 48 KB of dQ|dK|dV, double-
+// buffered in the room of the pairs' lo halves, and 96 KB of weights once per run
+// of tiles, where the other order loads 96 KB of weights per unit and 48 KB once per
+// run of chunks.  The kernel is bound by what passes between L2 and the SM: 128 KB of
+// reductions a unit at 38 GB/s per SM, and these loads.  Measured in the step: B4 T4096
+// d1024 H8 k2048 62 -> 59 us, B16 T1024 d1024 H64 k64 76 -> 72, B2 T8192 d1024
+// H32 k256 37.2 -> 36.3.
 // Warps: 0 TMA producer, 1 MMA issuer, 2 TMEM owner, 3 idle, 4-11 epilogue
 // (warp w: tile rows 32 (w % 4) .. +31, chunk columns 128 ((w - 4) / 4) ..).
 // Every wait is bounded.
@@ -43,9 +51,10 @@ constexpr int kWBytes = 256 * 128;   // one weight block of a chunk: 32 KB
 
 struct DxSmem {
     uint8_t a[3][2][kTileHalf];      // A pairs of the tile [j][hi / lo]: dQ, dK, dV, or AR
+                                     // (kWS: fp16 A_j of unit i in [j][i % 2])
     uint8_t w[kSlots][kWBytes];      // weight blocks
     uint8_t stage[8][4096];          // epilogue staging, one buffer per epilogue warp
-    uint64_t a_full[3], a_empty[3], w_full[kSlots], w_empty[kSlots], out_full[2], out_empty[2];
+    uint64_t a_full[6], a_empty[6], w_full[kSlots], w_empty[kSlots], out_full[2], out_empty[2];
     uint64_t drained;   // the MMA issuer's final drain
     uint32_t tmem;
     int abort;
@@ -79,7 +88,8 @@ __device__ __forceinline__ bool dwait(DxSmem &sm, uint64_t &bar, uint32_t parity
 
 // kOut = false: dX (three A matrices, K-major W_j blocks, plus dlogit W_r);
 // kOut = true: Y (one A matrix, AR; MN-major W_o chunks).
-template <bool kOut>
+// kWS (dX with fp16 rows): weights stay for a run of tiles.
+template <bool kOut, bool kWS>
 __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __grid_constant__ DxParams p) {
     constexpr int NM = kOut ? 1 : 3;          // A matrices per tile
     constexpr int kLo = kOut ? 64 : 256;      // column of the lo half of a pair row
@@ -87,13 +97,14 @@ __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __gr
     DxSmem &sm = *reinterpret_cast<DxSmem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // this CTA's units [u0, u1); unit u = (h * mt + tile) * nch + chunk
+    // this CTA's units [u0, u1); unit u = (h * mt + tile) * nch + chunk, or with kWS
+    // (h * nch + chunk) * mt + tile
     const long long u0 = p.units * blockIdx.x / gridDim.x;
     const long long u1 = p.units * (blockIdx.x + 1) / gridDim.x;
     const int nu = (int)(u1 - u0);
 
     if (threadIdx.x == 0) {
-        for (int j = 0; j < NM; ++j) {
+        for (int j = 0; j < (kWS ? 2 * NM : NM); ++j) {
             mbar_init(smem_u32(&sm.a_full[j]), 1);
             mbar_init(smem_u32(&sm.a_empty[j]), 1);
         }
@@ -120,8 +131,46 @@ __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __gr
     pdl_wait();  // the A pairs (and dlogit) come from earlier kernels
     span_begin(p.span);
 
+    // unit u with kWS
+    auto at = [&](long long u, int &h, int &c, int &tile) {
+        const long long run = u / p.mt;
+        tile = (int)(u - run * p.mt);
+        h = (int)(run / p.nch);
+        c = (int)(run - (long long)h * p.nch);
+    };
     if (warp == 0) {
-        if (lane == 0) {
+        if (kWS && lane == 0) {
+            int runs = 0, na[3] = {0, 0, 0}, nwl[3] = {0, 0, 0};   // runs started; loads issued
+            bool ok = true;
+            for (int i = 0; i < nu && ok; ++i) {
+                int h, c, tile;
+                at(u0 + i, h, c, tile);
+                const bool fresh = i == 0 || tile == 0;
+                for (int j = 0; j < NM; ++j) {
+                    if (fresh) {
+                        // W_j of the previous run frees once its last j-products end
+                        if (!(ok = dwait(sm, sm.w_empty[j], (runs & 1) ^ 1, p.status))) break;
+                        const uint32_t fb = smem_u32(&sm.w_full[j]);
+                        mbar_expect_tx(fb, kWBytes);
+                        tma_load_3d(smem_u32(sm.w[j]), &p.mW[j], fb, 0, c * kChunk, h);
+                        ++nwl[j];
+                    }
+                    const int ab = 2 * j + (i & 1);
+                    if (!(ok = dwait(sm, sm.a_empty[ab], ((i >> 1) & 1) ^ 1, p.status))) break;
+                    const uint32_t fb = smem_u32(&sm.a_full[ab]);
+                    mbar_expect_tx(fb, kTileHalf);
+                    tma_load_3d(smem_u32(sm.a[j][i & 1]), &p.mA, fb, 64 * j, tile * 128, h);
+                    ++na[j];
+                }
+                if (fresh) ++runs;
+            }
+            // drain: the last load of every weight block and A buffer has landed
+            for (int j = 0; j < NM; ++j) {
+                if (nwl[j] > 0) drain_phase(smem_u32(&sm.w_full[j]), (nwl[j] - 1) & 1);
+                for (int i = max(0, na[j] - 2); i < na[j]; ++i)
+                    drain_phase(smem_u32(&sm.a_full[2 * j + (i & 1)]), (i >> 1) & 1);
+            }
+        } else if (lane == 0) {
             int ntile = 0;  // tiles started so far
             int nw = 0;     // weight-block loads issued
             int na[3] = {0, 0, 0};   // A_j loads issued
@@ -174,7 +223,31 @@ __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __gr
             const int halves = p.f16 ? 1 : 2;
             bool ok = true;
             int ntile = 0;
-            for (int i = 0; i < nu && ok; ++i) {
+            for (int i = 0; kWS && i < nu && ok; ++i) {
+                int h, c, tile;
+                at(u0 + i, h, c, tile);
+                const int buf = i & 1;
+                const bool fresh = i == 0 || tile == 0;
+                const bool last = tile == p.mt - 1 || i == nu - 1;   // the run's last unit here
+                if (i >= 2 && !(ok = dwait(sm, sm.out_empty[buf], ((i >> 1) - 1) & 1, p.status))) break;
+                for (int j = 0; j < NM && ok; ++j) {
+                    if (fresh && !(ok = dwait(sm, sm.w_full[j], ntile & 1, p.status))) break;
+                    if (!(ok = dwait(sm, sm.a_full[2 * j + buf], (i >> 1) & 1, p.status))) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_bf16(tmem + 256 * buf,
+                                 smem_desc_sw128(smem_u32(sm.a[j][buf]) + kk * 32, 16, 1024),
+                                 smem_desc_sw128(smem_u32(sm.w[j]) + kk * 32, 16, 1024), idX,
+                                 (j > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit(smem_u32(&sm.a_empty[2 * j + buf]));
+                    if (last) mma_commit(smem_u32(&sm.w_empty[j]));
+                }
+                if (!ok) break;
+                mma_commit(smem_u32(&sm.out_full[buf]));
+                if (fresh) ++ntile;   // runs started
+            }
+            for (int i = 0; !kWS && i < nu && ok; ++i) {
                 const long long u = u0 + i;
                 const int c = (int)(u % p.nch), buf = i & 1;
                 const bool fresh = i == 0 || c == 0;
@@ -222,10 +295,18 @@ __global__ void __launch_bounds__(kThreads, 1) scatter_product_kernel(const __gr
         float my_dl = 0.f;   // its dlogit (dX)
         for (int i = 0; i < nu; ++i) {
             const long long u = u0 + i;
-            const int c = (int)(u % p.nch), buf = i & 1;
-            const long long tile = u / p.nch;
-            const int h = (int)(tile / p.mt), m0 = (int)(tile % p.mt) * 128;
-            if (i == 0 || c == 0) {
+            const int buf = i & 1;
+            int h, c, m0;
+            if constexpr (kWS) {
+                at(u, h, c, m0);
+                m0 *= 128;
+            } else {
+                c = (int)(u % p.nch);
+                const long long tile = u / p.nch;
+                h = (int)(tile / p.mt);
+                m0 = (int)(tile % p.mt) * 128;
+            }
+            if (kWS || i == 0 || c == 0) {
                 const int m = m0 + q * 32 + lane;
                 my_row = m < p.Mtok ? p.gidx[(size_t)h * p.Mtok + m] : -1;
                 if (!kOut) my_dl = m < p.Mtok ? p.dlogit[(size_t)h * p.Mtok + m] : 0.f;
@@ -284,7 +365,7 @@ bool map3(CUtensorMap *m, const void *base, uint64_t H, uint64_t rows, uint64_t 
     return tmap_bf16(m, base, 3, dims, strides, box);
 }
 
-template <bool kOut>
+template <bool kOut, bool kWS>
 cudaError_t launch_scatter_product(DxParams &p, const Dims &dm, cudaStream_t s) {
     const int Mtok = dm.B * dm.k;
     p.Mtok = Mtok;
@@ -293,14 +374,14 @@ cudaError_t launch_scatter_product(DxParams &p, const Dims &dm, cudaStream_t s) 
     p.nch = (dm.d + kChunk - 1) / kChunk;
     p.units = (long long)dm.H * p.mt * p.nch;
     p.span = active_span();
-    const cudaError_t attr = allow_smem((const void *)scatter_product_kernel<kOut>, kSmem);
+    const cudaError_t attr = allow_smem((const void *)scatter_product_kernel<kOut, kWS>, kSmem);
     if (attr != cudaSuccess) return attr;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const long long grid = p.units < sms ? p.units : sms;
-    e = launch_pdl(scatter_product_kernel<kOut>, dim3((unsigned)grid), dim3(kThreads), kSmem, s, p);
+    e = launch_pdl(scatter_product_kernel<kOut, kWS>, dim3((unsigned)grid), dim3(kThreads), kSmem, s, p);
     note_launches(1);
     return e;
 }
@@ -326,7 +407,12 @@ cudaError_t tc_dx(const Dims &dm, const void *Wq, const void *Wk, const void *Wv
     p.WrT = sv.WrT;
     p.dX = dX;
     p.status = sv.status;
-    return launch_scatter_product<false>(p, dm, s);
+    // fp16 rows: the order that loads less per unit, 48 KB + 96 KB / (tiles per head)
+    // or 96 KB + 48 KB / (chunks per tile)
+    const int mt = (Mtok + 127) / 128, nch = (dm.d + kChunk - 1) / kChunk;
+    if (p.f16 && 48 * nch * mt + 96 * nch < 96 * nch * mt + 48 * mt)
+        return launch_scatter_product<false, true>(p, dm, s);
+    return launch_scatter_product<false, false>(p, dm, s);
 }
 
 cudaError_t tc_out_scatter(const Dims &dm, const void *Wo, const Saved &sv, float *Y,
@@ -344,7 +430,7 @@ cudaError_t tc_out_scatter(const Dims &dm, const void *Wo, const Saved &sv, floa
     p.gidx = sv.gidx;
     p.dX = Y;
     p.status = sv.status;
-    return launch_scatter_product<true>(p, dm, s);
+    return launch_scatter_product<true, false>(p, dm, s);
 }
 
 }  // namespace mosa
