@@ -251,15 +251,15 @@ def traffic_for(stage, cfg_name):
 
 # Kernel name (as ncu prints it) -> bench stage.
 KERNEL_STAGE = [("tc_gemm_kernel<5>", "router"), ("tc_gemm_kernel<(int)5>", "router"),
-                ("pad_wr_kernel", "router"),
-                ("topk_select", "select"), ("tc_gemm_kernel<0>", "qkv"),
+                ("pad_wr_kernel", "router"), ("router_rows", "router"),
+                ("topk_select", "select"), ("topk_long", "select"), ("tc_gemm_kernel<0>", "qkv"),
                 ("tc_gemm_kernel<(int)0>", "qkv"), ("attn_fwd", "attn_fwd"),
                 ("tc_gemm_kernel<2>", "out_bwd"), ("tc_gemm_kernel<(int)2>", "out_bwd"),
                 ("attn_bwd", "attn_bwd"), ("dq_finish", "attn_bwd"),
-                ("scatter_product_kernel<0>", "in_bwd"), ("scatter_product_kernel<false>", "in_bwd"),
-                ("scatter_product_kernel<(bool)0>", "in_bwd"),
-                ("scatter_product_kernel<1>", "out"), ("scatter_product_kernel<true>", "out"),
-                ("scatter_product_kernel<(bool)1>", "out"),
+                ("scatter_product_kernel<0", "in_bwd"), ("scatter_product_kernel<false", "in_bwd"),
+                ("scatter_product_kernel<(bool)0", "in_bwd"),
+                ("scatter_product_kernel<1", "out"), ("scatter_product_kernel<true", "out"),
+                ("scatter_product_kernel<(bool)1", "out"),
                 ("head_sum_kernel<true>", "out"), ("head_sum_kernel<(bool)1>", "out"),
                 ("head_sum_kernel<1>", "out"),
                 ("tc_gemm_kernel<4>", "w_bwd"), ("tc_gemm_kernel<(int)4>", "w_bwd"),
@@ -286,7 +286,7 @@ def ingest_ncu(csv_path, cfg_name):
         lines = [l for l in f if not l.startswith("==")]
     for row in csv.DictReader(lines):
         name, metric = row.get("Kernel Name", ""), row.get("Metric Name", "")
-        if "topk_select" in name:
+        if "topk_select" in name or "topk_long" in name:
             steps.add(row["ID"])
         if metric not in ("dram__bytes_read.sum", "dram__bytes_write.sum"):
             continue
