@@ -12,6 +12,7 @@
 // when a tensor's address is not 16-byte aligned.
 // dQ|dK|dV rows have 4 h' columns: 3 h' of gradients, then dlogit (bf16: its
 // pair at column 3 h' and the pair of what that rounded off at 3 h' + 1).
+#include <algorithm>
 #include <cstdlib>
 #include <initializer_list>
 #include <type_traits>
@@ -89,11 +90,11 @@ struct QkvOp {
     }
     __device__ float a(int g, int m, int c) const { return to_f32(A[(size_t)a_row(g, m) * K + c]); }
     __device__ float b(int g, int c, int n) const { return to_f32(*b_ptr(g, c, n)); }
-    __device__ void store(int g, int m, int n, float v, bool) const {
+    __device__ void store(int g, int m, int n, float v, int) const {
         const int w = n >> lg, p = n & (hp - 1);
         Inter<TS>::st(w == 0 ? Q : (w == 1 ? Kp : V), (size_t)g * M + m, hp, p, v);
     }
-    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+    __device__ void store4(int g, int m, int n, const float4 &v, int) const {
         const int w = n >> lg, p = n & (hp - 1);
         st_inter4<T>(w == 0 ? Q : (w == 1 ? Kp : V), (size_t)g * M + m, hp, p, v);
     }
@@ -117,13 +118,21 @@ struct OutOp {
     __device__ const T *b_ptr(int g, int p, int n) const { return Wo + ((size_t)g * K + p) * N + n; }
     __device__ float a(int g, int m, int p) const { return Inter<TS>::ld(A, (size_t)g * M + m, K, p); }
     __device__ float b(int g, int p, int n) const { return to_f32(*b_ptr(g, p, n)); }
-    __device__ void store(int g, int m, int n, float v, bool) const {
+    __device__ void store(int g, int m, int n, float v, int) const {
         atomicAdd(Y + (size_t)gidx[(size_t)g * M + m] * N + n, v);
     }
-    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+    __device__ void store4(int g, int m, int n, const float4 &v, int) const {
         tc::red_add_v4(Y + (size_t)gidx[(size_t)g * M + m] * N + n, v.x, v.y, v.z, v.w);
     }
 };
+
+// G's reduction splits: split 0 (or the only one) goes to G, split j to the j-th h'
+// columns of the rows of dQ|dK|dV (4 h' fp32 columns), which the attention backward
+// writes later; out_bwd_rows_kernel adds them up, so G stays one fixed sum.
+constexpr int kGSplits = 5;
+__device__ __forceinline__ float *g_part(float *G, void *dQKV, size_t row, int hp, int sp) {
+    return sp <= 0 ? G + row * hp : static_cast<float *>(dQKV) + row * 4 * hp + (sp - 1) * hp;
+}
 
 template <class T>
 struct OutBwdGOp {
@@ -137,14 +146,18 @@ struct OutBwdGOp {
     const T *Wo;
     const int32_t *gidx;
     float *G;
+    void *dQKV;
     int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
     __device__ int a_row(int g, int m) const { return gidx[(size_t)g * M + m]; }
     __device__ const T *b_ptr(int g, int n, int c) const { return Wo + ((size_t)g * N + n) * K + c; }
     __device__ float a(int g, int m, int c) const { return to_f32(A[(size_t)a_row(g, m) * K + c]); }
     __device__ float b(int g, int c, int n) const { return to_f32(*b_ptr(g, n, c)); }
-    __device__ void store(int g, int m, int n, float v, bool) const { G[((size_t)g * M + m) * N + n] = v; }
-    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
-        *reinterpret_cast<float4 *>(G + ((size_t)g * M + m) * N + n) = v;
+    __device__ float *row(int g, int m, int sp) const {
+        return g_part(G, dQKV, (size_t)g * M + m, N, sp);
+    }
+    __device__ void store(int g, int m, int n, float v, int sp) const { row(g, m, sp)[n] = v; }
+    __device__ void store4(int g, int m, int n, const float4 &v, int sp) const {
+        *reinterpret_cast<float4 *>(row(g, m, sp) + n) = v;
     }
 };
 
@@ -169,10 +182,10 @@ struct OutBwdWOp {
     }
     __device__ float a(int g, int c, int m) const { return to_f32(A[(size_t)a_row(g, m) * M + c]); }
     __device__ float b(int g, int m, int p) const { return Inter<TS>::ld(AR, (size_t)g * K + m, N, p); }
-    __device__ void store(int g, int c, int p, float v, bool add) const {
-        put1(dWo + ((size_t)g * N + p) * M + c, v, add);
+    __device__ void store(int g, int c, int p, float v, int sp) const {
+        put1(dWo + ((size_t)g * N + p) * M + c, v, sp >= 0);
     }
-    __device__ void store4(int, int, int, const float4 &, bool) const {}
+    __device__ void store4(int, int, int, const float4 &, int) const {}
 };
 
 template <class T>
@@ -198,12 +211,12 @@ struct InBwdOp {
     }
     __device__ float a(int g, int m, int kk) const { return Inter<TS>::ld(A, (size_t)g * M + m, 4 * hp, kk); }
     __device__ float b(int g, int kk, int n) const { return to_f32(*b_ptr(g, n, kk)); }
-    __device__ void store(int g, int m, int n, float v, bool) const {
+    __device__ void store(int g, int m, int n, float v, int) const {
         const size_t row = (size_t)g * M + m;
         v = fmaf(dlogit[row], to_f32(Wr[(size_t)n * H + g]), v);
         atomicAdd(dX + (size_t)gidx[row] * N + n, v);
     }
-    __device__ void store4(int g, int m, int n, const float4 &v, bool) const {
+    __device__ void store4(int g, int m, int n, const float4 &v, int) const {
         const size_t row = (size_t)g * M + m;
         const float dl = dlogit[row];
         const T *w = Wr + (size_t)n * H + g;
@@ -245,17 +258,17 @@ struct WBwdOp {
         const int w = n >> lg, p = n & (hp - 1);
         return (w == 0 ? dWq : (w == 1 ? dWk : dWv)) + ((size_t)g * M + c) * hp + p;
     }
-    __device__ void store(int g, int c, int n, float v, bool add) const {
+    __device__ void store(int g, int c, int n, float v, int sp) const {
         if (n < 3 * hp)
-            put1(dst(g, c, n), v, add);
+            put1(dst(g, c, n), v, sp >= 0);
         else if (n == 3 * hp)
-            put1(dWr + (size_t)c * H + g, v, add);
+            put1(dWr + (size_t)c * H + g, v, sp >= 0);
     }
-    __device__ void store4(int g, int c, int n, const float4 &v, bool add) const {
+    __device__ void store4(int g, int c, int n, const float4 &v, int sp) const {
         if (n < 3 * hp)
-            put4(dst(g, c, n), v, add);
+            put4(dst(g, c, n), v, sp >= 0);
         else
-            put1(dWr + (size_t)c * H + g, kExtra == 2 ? v.x + v.y : v.x, add);
+            put1(dWr + (size_t)c * H + g, kExtra == 2 ? v.x + v.y : v.x, sp >= 0);
     }
 };
 
@@ -263,10 +276,10 @@ struct WBwdOp {
 // D = rowsum(dA o A), dlogit = dr r (1 - r).
 // (Pointers without __restrict__: see attn_fwd_simt_kernel.)
 template <class TS>
-__global__ void out_bwd_rows_kernel(const float *G, const float *A,
+__global__ void out_bwd_rows_kernel(float *G, const float *A,
                                     const float *rsel, void *dA,
                                     float *Dd, float *dlogit,
-                                    void *dQKV, long long rows, int hp) {
+                                    void *dQKV, long long rows, int hp, int splits) {
     tc::pdl_wait();
     const long long row = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
@@ -274,7 +287,8 @@ __global__ void out_bwd_rows_kernel(const float *G, const float *A,
     const float r = rsel[row];
     float dr = 0.f, dd = 0.f;
     for (int p = lane; p < hp; p += 32) {
-        const float g = G[row * hp + p];
+        float g = G[row * hp + p];
+        for (int j = 1; j < splits; ++j) g += g_part(G, dQKV, row, hp, j)[p];
         const float a = A[row * hp + p];
         dr = fmaf(a, g, dr);
         const float da = r * g;
@@ -351,22 +365,35 @@ cudaError_t out_t(const Dims &dm, const void *Wo, const Saved &sv, float *Y, cud
     return product(op, dm.H, 1, use_split() && aligned16({Wo, Y}), sv, s);
 }
 
+// G has one column tile per 128 rows: as many reduction splits as the 152 SMs have
+// room for, each of at least three K blocks and none of them empty.
+// fp32 at B4 T1000 d768 H12 k125, 48 tiles: 28 -> 15 us on 144 CTAs, its step 225 -> 210.
+// bf16 storage, whose K blocks are only copied, keeps one: at B4 T1024 d1024 H16 h'=128
+// k128, 64 tiles, two splits took 17 -> 13 us here and the step 285.6 -> 286.5.
+int g_split_count(int M, int N, int K, int groups) {
+    const int tiles = (M + 127) / 128 * ((N + 127) / 128) * groups, nkb = (K + 63) / 64;
+    const int sp = std::max(1, std::min({kGSplits, 152 / tiles, nkb / 3}));
+    const int per = (nkb + sp - 1) / sp;
+    return (nkb + per - 1) / per;
+}
+
 template <class T>
 cudaError_t out_bwd_t(const Dims &dm, const void *Wo, const void *dY, const Saved &sv,
                       float *dWo, cudaStream_t s) {
     using TS = typename InterOf<T>::type;
     const bool split = use_split() && aligned16({Wo, dY, dWo});
     const int Mtok = dm.B * dm.k;
-    OutBwdGOp<T> g{Mtok, dm.hp, dm.d, (const T *)dY, (const T *)Wo, sv.gidx, sv.G};
+    OutBwdGOp<T> g{Mtok, dm.hp, dm.d, (const T *)dY, (const T *)Wo, sv.gidx, sv.G, sv.dQKV};
     g.lda = dm.d;
     g.ldb = dm.d;
-    cudaError_t e = product(g, dm.H, 1, split, sv, s);
+    const int gsplits = split && sizeof(T) == 4 ? g_split_count(Mtok, dm.hp, dm.d, dm.H) : 1;
+    cudaError_t e = product(g, dm.H, gsplits, split, sv, s);
     if (e != cudaSuccess) return e;
     const long long rows = dm.rows();
     const int warps = 8;
     e = launch_pdl(out_bwd_rows_kernel<TS>, dim3((unsigned)((rows + warps - 1) / warps)),
-                   dim3(warps * 32), 0, s, (const float *)sv.G, (const float *)sv.A,
-                   (const float *)sv.rsel, sv.dA, sv.Dd, sv.dlogit, sv.dQKV, rows, dm.hp);
+                   dim3(warps * 32), 0, s, sv.G, (const float *)sv.A,
+                   (const float *)sv.rsel, sv.dA, sv.Dd, sv.dlogit, sv.dQKV, rows, dm.hp, gsplits);
     note_launches(1);
     if (e != cudaSuccess) return e;
     const int splits = split ? split_count(dm.d, dm.hp, Mtok, dm.H) : 1;

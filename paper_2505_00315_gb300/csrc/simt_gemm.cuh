@@ -5,7 +5,7 @@
 // For every group g (blockIdx.z) it computes C[g](m,n) = sum_kk A(g,m,kk) B(g,kk,n)
 // for 0 <= m < op.M, 0 <= n < op.N, 0 <= kk < op.K, reading elements through
 // op.a(g,m,kk) / op.b(g,kk,n) and handing each result to
-// op.store(g,m,n,acc,false) (true: add to what other reduction splits store).
+// op.store(g,m,n,acc,-1) (the one reduction split there is).
 // The functors carry the gathers (rows chosen by a head), transposes and
 // scatter-adds of the MoSA steps.
 #pragma once
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kSimtThreads) simt_gemm_kernel(Op op) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int m = m0 + tm + i, n = n0 + tn + j;
-            if (m < op.M && n < op.N) op.store(g, m, n, acc[i][j], false);
+            if (m < op.M && n < op.N) op.store(g, m, n, acc[i][j], -1);
         }
 }
 

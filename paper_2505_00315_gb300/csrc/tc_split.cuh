@@ -55,8 +55,8 @@ namespace mosa {
 //   a_row(g, r)           source row of A for strided index r (r < M or r < K)
 //   b_ptr(g, r, c)        eight contiguous elements of B: strided index r (k if kBMN,
 //                         else n), contiguous index c; linear in r with stride ldb; b_lo as a_lo
-//   store(g, m, n, v, add)     one result; add: several reduction splits add up
-//   store4(g, m, n, v4, add)   four consecutive columns (not kTrans)
+//   store(g, m, n, v, sp)      one result of reduction split sp (-1: the only one)
+//   store4(g, m, n, v4, sp)    four consecutive columns (not kTrans)
 struct SplitArgs {
     int bn;        // tile width, a multiple of 16, <= 128
     int nt, mt;    // column and row tiles of a group
@@ -113,16 +113,17 @@ __device__ __forceinline__ void split3(const float4 &x, const float4 &y, uint4 (
 
 // Tile t: column tiles fastest (neighbouring CTAs read the same rows of A).
 struct SplitTile {
-    int g, m0, n0, kb0, nkb;
+    int g, m0, n0, kb0, nkb, sp;   // sp: reduction split, -1 where there is only one
     __device__ __forceinline__ SplitTile(const SplitArgs &sa, unsigned t) {
-        unsigned n = 0, m = 0, sp = 0;   // (a division by 1 is not worth its instructions)
+        unsigned n = 0, m = 0;   // (a division by 1 is not worth its instructions)
         if (sa.nt > 1) n = t % (unsigned)sa.nt, t /= (unsigned)sa.nt;
         if (sa.mt > 1) m = t % (unsigned)sa.mt, t /= (unsigned)sa.mt;
         kb0 = 0;
         nkb = sa.nkb;
+        sp = -1;
         if (sa.splits > 1) {
-            sp = t % (unsigned)sa.splits, t /= (unsigned)sa.splits;
-            kb0 = (int)sp * sa.per;
+            sp = (int)(t % (unsigned)sa.splits), t /= (unsigned)sa.splits;
+            kb0 = sp * sa.per;
             nkb = max(0, min(sa.nkb, kb0 + sa.per) - kb0);
         }
         g = (int)t;
@@ -460,7 +461,6 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
             if (tile + step >= sa.tiles) pdl_trigger();
             const int nb = tl.n0 + 64 * hf, n_end = min(op.N, tl.n0 + sa.bn);
             const int m = tl.m0 + q * 32 + lane;
-            const bool add = sa.splits > 1;
             if constexpr (kF32) {
                 bool nan = false;
 #pragma unroll
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
                             float acc = 0.f;
                             for (int k = tl.kb0 * 64; k < k_end; ++k)
                                 acc = fmaf(op.a(tl.g, m, k), op.b(tl.g, k, n), acc);
-                            op.store(tl.g, m, n, acc, add);
+                            op.store(tl.g, m, n, acc, tl.sp);
                         }
                     continue;
                 }
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
                 if (m < op.M) {
 #pragma unroll
                     for (int j = 0; j < 64; ++j)
-                        if (nb + j < n_end) op.store(tl.g, m, nb + j, v[j], add);
+                        if (nb + j < n_end) op.store(tl.g, m, nb + j, v[j], tl.sp);
                 }
             } else {
                 // through a 4 KB per-warp buffer, so that every store or reduction
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
                         const int rl = (lane >> 3) + 4 * i, mr = tl.m0 + q * 32 + rl;
                         const int n = nb + c0 + 4 * (lane & 7);
                         const float4 x = *reinterpret_cast<const float4 *>(xb + xoff128(rl, lane & 7));
-                        if (mr < op.M && n < n_end) op.store4(tl.g, mr, n, x, add);
+                        if (mr < op.M && n < n_end) op.store4(tl.g, mr, n, x, tl.sp);
                     }
                     __syncwarp();
                 }
@@ -513,8 +513,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
     }
 }
 
-// Launches op over `groups` groups; splits as chosen by split_count (the
-// caller zeroes the output first where it is above 1).
+// Launches op over `groups` groups; splits as chosen by split_count (where it is above
+// 1 and the op's splits add up in place, the caller zeroes the output first).
 template <class Op>
 inline cudaError_t launch_split_gemm(const Op &op, int groups, int splits, uint32_t *status,
                                      cudaStream_t stream) {

@@ -189,6 +189,23 @@ def test_plane_products_many_tiles_parity(cfg):
         assert_close(name, g[gname], ref[name], cfg.dtype)
 
 
+# dY W_o^T of fp32 layers in reduction splits whose partial sums the row terms add up:
+# five with a last K block of 8, two of unequal length
+@pytest.mark.parametrize("cfg", [
+    W.MosaConfig("g_five_splits", B=2, T=90, d=1032, H=3, hp=16, k=40, dtype="f32", seed=78),
+    W.MosaConfig("g_two_splits", B=2, T=210, d=392, H=5, hp=128, k=130, dtype="f32", seed=79),
+], ids=lambda c: c.name)
+def test_f32_row_terms_over_reduction_splits_parity(cfg):
+    x = W.make_inputs(cfg)
+    _, I, _, _ = oracle.forward(x["X"], *weights(x), k=cfg.k)
+    g = run_layer(cfg, x, backward=True)
+    np.testing.assert_array_equal(g["I"], I)
+    ref = oracle.backward(x["X"], *weights(x), I=I, dY=x["dY"])
+    for name in ("dX", "dWr", "dWq", "dWk", "dWv", "dWo"):
+        gname = name[:2] + "_" + name[2:].lower() if name != "dX" else "dX"
+        assert_close(name, g[gname], ref[name], cfg.dtype)
+
+
 # Fused forward with few tiles: a tile's output columns shared by several CTAs, with
 # a last column block cut short and one block more than CTAs
 @pytest.mark.parametrize("cfg", [
