@@ -287,7 +287,9 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
             }
             for (int n = 0; have; ++n) {
                 const int s = n % S;
-                if (!mbar_wait(smem_u32(&empty[s]), ((n / S) & 1) ^ 1) || *(volatile int *)s_abort) {
+                // (warp-uniform: the row shuffles are warp-collective)
+                if (__any_sync(0xffffffffu, !mbar_wait(smem_u32(&empty[s]), ((n / S) & 1) ^ 1) ||
+                                                *(volatile int *)s_abort)) {
                     give_up();
                     break;
                 }
@@ -326,7 +328,9 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
             int landed = 0, issued = 0;
             for (int n = 0; w.tile < sa.tiles; ++n) {
                 const int s = n % S;
-                if (!mbar_wait(smem_u32(&empty[s]), ((n / S) & 1) ^ 1) || *(volatile int *)s_abort) {
+                // (warp-uniform: the row shuffles are warp-collective)
+                if (__any_sync(0xffffffffu, !mbar_wait(smem_u32(&empty[s]), ((n / S) & 1) ^ 1) ||
+                                                *(volatile int *)s_abort)) {
                     give_up();
                     break;
                 }
