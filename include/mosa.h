@@ -57,7 +57,9 @@
  *     values (11-bit significand) for k > 128, one MMA per product: a value
  *     beyond the fp16 range (|v| > 65504) is reported as MOSA_ERR_RANGE by
  *     mosa_check_status() rather than passed on silently.  With fp32 storage
- *     every intermediate is fp32.
+ *     every intermediate is fp32; the products run on the tensor cores
+ *     with every fp32 operand cut into three bf16 parts (an exact cut), and are as close to
+ *     64-bit results as fp32 multiply-add chains.
  *   - Tokens tied on the router score are taken lowest index first.
  *   - NaN inputs give undefined results (but no out-of-bounds access).
  *   - Errors: a call that returns anything but MOSA_OK has launched nothing.

@@ -89,10 +89,11 @@ struct Saved {
     void *dA;           // [H,B*k,hp] gradient of A, intermediate
     float *dlogit;      // [H,B*k]   gradient of the router logit
     float *Dd;          // [H,B*k]   rowsum(dA o A)
-    void *dQKV;         // [H,B*k,3hp] dQ | dK | dV, intermediate (tensor-core path:
+    void *dQKV;         // [H,B*k,4hp] dQ | dK | dV | dlogit, intermediate (tensor-core path:
                         // [H,B*k,512] bf16 pair dQ|dK|dV|dlogit,0.. hi then lo)
-    float *G;           // [H,B*k,hp] dY[I] W_o^T (fp32, CUDA-core path); on the
-                        // tensor-core path with k > 128 the fp32 dQ accumulator
+    float *G;           // [H,B*k,hp] dY[I] W_o^T (fp32; fp32 storage and head sizes other
+                        // than 64); on the tensor-core path with k > 128 the fp32 dQ
+                        // accumulator
     float *WrT;         // [H,d] fp32 transpose of W_r (tensor-core dX epilogue)
     void *Wr64;         // [d, H rounded up to 64] bf16 W_r with zero columns past H
                         // (tensor-core router, H % 64 != 0)

@@ -144,7 +144,8 @@ cudaError_t launch_w_bwd(const Dims &dm, const void *X, const Saved &sv, float *
 // ---- tensor-core path (tc_gemm.cu): bf16 inputs, head size 64 ----
 bool tc_supported(const Dims &dm);
 // False when the environment variable MOSA_FORCE_SIMT is set to a non-zero
-// value: the projections then run on the CUDA cores for every shape.
+// value: the projections then run on the CUDA cores for every shape (else on the tensor
+// cores, those of fp32 storage and other head sizes through bf16 planes).
 bool use_split();
 // True when the tensor-core kernels serve this shape (false also when the
 // environment variable MOSA_FORCE_SIMT is set to a non-zero value).

@@ -110,9 +110,9 @@ constexpr uint32_t kBackwardStages = (1u << kStageOutBwd) | (1u << kStageAttnBwd
 // ------------------------------------------------ concurrent branches
 // On the tensor-core path independent kernels run on a second, internal
 // stream joined back with events (graph branches when captured):
-//   forward:  zeroing Y and (fp16 attention path) the fp16 copies of X and
-//             W_q|W_k|W_v run beside TopK (forked after the router, joined
-//             before the output product);
+//   forward:  zeroing Y and the fp16 copies of X and W_q|W_k|W_v (where the
+//             backward reads them) run beside TopK (forked after the router,
+//             joined before the output product);
 //   backward: dW_o, the W_r transpose and (except on the fp16 path, where
 //             the attention backward does it) the zeroing of dX run beside
 //             G -> attention backward; then dX and dW run side by side.
