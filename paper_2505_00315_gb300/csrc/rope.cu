@@ -91,8 +91,7 @@ struct Oct<SplitBF16> {
 // of two (lg = log2).
 template <class TS>
 __global__ void rope_rows_kernel(void *p0, void *p1, int col0_0, int col0_1, int cols, int lg,
-                                 long long rows, const int32_t *__restrict__ gidx, RopeTable tab,
-                                 float dir) {
+                                 long long rows, const int32_t *gidx, RopeTable tab, float dir) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long row = i >> (lg + 1);

@@ -613,10 +613,8 @@ topk_long_kernel(const float *scores, int T, int k, int32_t *I,
     }
 }
 
-__global__ void indices_to_rows_kernel(const int32_t *__restrict__ I,
-                                       const float *__restrict__ rsel, int B, int H, int T,
-                                       int k, int32_t *__restrict__ gidx,
-                                       float *__restrict__ rsel_hm, uint32_t *status) {
+__global__ void indices_to_rows_kernel(const int32_t *I, const float *rsel, int B, int H, int T,
+                                       int k, int32_t *gidx, float *rsel_hm, uint32_t *status) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int row = blockIdx.x;  // b*H + h
     const int hh = row % H, bb = row / H;

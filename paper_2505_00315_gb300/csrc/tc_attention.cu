@@ -663,8 +663,8 @@ __global__ void __launch_bounds__(kBT, 1) attn_bwd_tc_kernel(const __grid_consta
         auto row_terms = [&](int i, float &l2, float &dd) {
             const int qi = (jt + i) * 128 + r;
             const bool v = i < nb && qi < p.k;
-            l2 = v ? __ldg(p.lse + base + qi) * 1.4426950408889634f : 0.f;
-            dd = v ? __ldg(p.Dd + base + qi) : 0.f;
+            l2 = v ? p.lse[base + qi] * 1.4426950408889634f : 0.f;
+            dd = v ? p.Dd[base + qi] : 0.f;
         };
         float l2n, ddn;
         row_terms(0, l2n, ddn);
@@ -776,10 +776,10 @@ __global__ void __launch_bounds__(kBT, 1) attn_bwd_tc_kernel(const __grid_consta
 // dQ from its fp32 accumulator into columns 0..63 of the dQ|dK|dV|dlogit rows,
 // eight columns per thread (two 16-byte loads): as a bf16 pair ([hi 256 | lo
 // 256] rows), or (f16) as fp16 rows of 256 (one 16-byte store), turned back by
-// RoPE first when asked (gidx, rope).
-__global__ void dq_finish_kernel(const float *__restrict__ dQacc, bf16 *__restrict__ dQKV, size_t rows,
-                                 int f16, const int32_t *__restrict__ gidx, int rope, int T,
-                                 RopeTable tab, uint32_t *status, unsigned long long *span) {
+// RoPE first when asked (gidx, rope).  (Plain loads after the wait: see pdl_wait.)
+__global__ void dq_finish_kernel(const float *dQacc, bf16 *dQKV, size_t rows, int f16,
+                                 const int32_t *gidx, int rope, int T, RopeTable tab,
+                                 uint32_t *status, unsigned long long *span) {
     pdl_trigger();  // the next kernel (zeroing dX) may run beside this one
     pdl_wait();
     span_begin(span);

@@ -158,7 +158,9 @@ __device__ __forceinline__ void cp_async_wait() {
 // ------------------------------------------- programmatic dependent launch
 // A kernel launched with programmatic stream serialization may start while
 // its predecessor is still running; it must call pdl_wait() before reading
-// anything the predecessor writes.  pdl_trigger() lets the successor launch.
+// anything the predecessor writes, and read that with plain loads: one that the
+// compiler may treat as constant data (__ldg, or through const __restrict__) can
+// move ahead of the wait, as it did in TopK.  pdl_trigger() lets the successor launch.
 // Both are no-ops for kernels launched without the attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {

@@ -950,8 +950,7 @@ __global__ void __launch_bounds__(kSideCta) zero_kernel(float4 *p, size_t n4) {
     if (i < n4) p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void transpose_wr_kernel(const bf16 *__restrict__ Wr, float *__restrict__ WrT, int d,
-                                    int H) {
+__global__ void transpose_wr_kernel(const bf16 *Wr, float *WrT, int d, int H) {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;  // element of WrT [H, d]
     if (i < d * H) {

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kHsThreads, 1) head_sum_kernel(const __grid_co
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int tt = t0 + sub + 16 * j;
-                pr[j] = tt < p.T ? __ldg(p.pos + (size_t)h * BT + (size_t)b * p.T + tt) : -1;
+                pr[j] = tt < p.T ? p.pos[(size_t)h * BT + (size_t)b * p.T + tt] : -1;
             }
         };
         int prow[8], pnext[8];
@@ -312,10 +312,10 @@ __global__ void __launch_bounds__(kHsThreads, 1) head_sum_kernel(const __grid_co
                 int pr[kHsMaxDlHeads];
 #pragma unroll
                 for (int h = 0; h < kHsMaxDlHeads; ++h)
-                    pr[h] = (h < p.H && tt < p.T) ? __ldg(p.pos + (size_t)h * BT + (size_t)b * p.T + tt) : -1;
+                    pr[h] = (h < p.H && tt < p.T) ? p.pos[(size_t)h * BT + (size_t)b * p.T + tt] : -1;
 #pragma unroll
                 for (int h = 0; h < kHsMaxDlHeads; ++h)
-                    sm.dl[r][h] = pr[h] >= 0 ? __ldg(p.dlogit + (size_t)h * p.Mtok + pr[h]) : 0.f;
+                    sm.dl[r][h] = pr[h] >= 0 ? p.dlogit[(size_t)h * p.Mtok + pr[h]] : 0.f;
                 __syncwarp();
             }
             const bool got = hwait(sm, sm.acc_full[buf], (i >> 1) & 1, p.status);
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kHsThreads, 1) head_sum_kernel(const __grid_co
                     val[rr] = *reinterpret_cast<const float4 *>(xb + xoff128((lane >> 3) + 4 * rr, cu));
                 if (!kOut && col < p.d) {
                     for (int h = 0; h < p.H; ++h) {
-                        const float4 w = __ldg(reinterpret_cast<const float4 *>(p.WrT + (size_t)h * p.d + col));
+                        const float4 w = *reinterpret_cast<const float4 *>(p.WrT + (size_t)h * p.d + col);
 #pragma unroll
                         for (int rr = 0; rr < 8; ++rr) {
                             const float dl = sm.dl[q * 32 + (lane >> 3) + 4 * rr][h];
