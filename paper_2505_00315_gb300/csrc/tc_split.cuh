@@ -3,20 +3,21 @@
 // storage, and bf16 storage with a head size other than 64.
 //
 // Every operand element is a sum of bf16 "planes": one for a bf16 input, two
-// for a stored bf16 hi/lo pair, three for an fp32 value (its significand cut
-// into three 8-bit parts, an exact decomposition: v = p0 + p1 + p2 with
-// p_i = the bf16 truncation of what the parts before it left).  The product of
+// for a stored bf16 hi/lo pair, three for an fp32 value: p0 = bf16(v), p1 = bf16(v - p0),
+// p2 = v - p0 - p1, each rounded to nearest, an exact cut (with v in [2^e, 2^(e+1)), p1 is at
+// most 2^(e-8), and p2 at most 2^(e-17) in steps of 2^(e-23)).  The product of
 // two operands is the sum of the plane products that matter: 1 (bf16 x bf16),
-// 2 (pair x bf16) or, for fp32 x fp32, the six of order up to 2^-16 (p0 q0,
-// p0 q1, p1 q0, p1 q1, p0 q2, p2 q0); what is left out is below 2^-23 of each
-// product, under the rounding of an fp32 multiply-add chain.  Each plane product
+// 2 (pair x bf16) or, for fp32 x fp32, the six of order up to 2^-17 (p0 q0,
+// p0 q1, p1 q0, p1 q1, p0 q2, p2 q0); what is left out is at most 2^-24 of each
+// product and of either sign, under the rounding of an fp32 multiply-add chain.  (Parts
+// cut off by truncation all have v's sign: they left out up to 2^-21, always
+// towards zero, and results were up to four times as far off as a chain's.)  Each plane product
 // of a K step is one MMA into the same accumulator, and the accumulator is
-// drained into fp32 registers every two or four steps (split_drain), so that the tensor
+// drained into fp32 registers after every 64-wide K block, so that the tensor
 // pipe's accumulation rounding acts on short partial sums only.
 //
-// A truncated non-finite fp32 input turns into NaN (inf - inf), and with it the whole
-// row or column of results it takes part in, where a plain product may give inf:
-// results around a NaN are computed again with plain fp32 multiply-adds.
+// Results around an infinity, or past the fp32 range, can come out as NaN where a plain
+// product is infinite: results around a NaN are computed again with plain fp32 multiply-adds.
 //
 // One CTA (544 threads) per SM walks over 128 x bn tiles (bn <= 128) of all groups:
 //   warps 0-7    drain: TMEM -> registers (four accumulators in turn), then the
@@ -76,36 +77,41 @@ template <class Op>
 constexpr bool split_f32() { return sizeof(typename Op::TA) == 4; }
 template <class Op>
 constexpr int split_stages() { return split_f32<Op>() ? 2 : (Op::kPA + Op::kPB == 2 ? 6 : 4); }
-// 16-wide K steps between drains: two for fp32, four (one K block) for bf16 inputs.
-// The tensor pipe does not round its accumulation to nearest: with four and sixteen
-// steps, errors against 64 bits were up to 6% (fp32, K = 128) and 4% (bf16, d =
-// 1024) above those of the multiply-add chains these products replace; with two and four
-// they are below them at every size measured (fp32 by 5 to 40%), for 1% and 4%
-// of these kernels' time.
-template <class Op>
-constexpr int split_drain() { return split_f32<Op>() ? 2 : 4; }
-constexpr int kSplitAcc = 4;   // accumulators (128 TMEM columns each)
+// Accumulators (128 TMEM columns each), one K block (four 16-wide steps) in each: the
+// tensor pipe does not round its accumulation to nearest, and with sixteen steps between
+// drains bf16 errors against 64 bits were up to 4% (d = 1024) above those of the
+// multiply-add chains that these products replace.  With four they are at or below them at
+// every size measured (fp32 by 15 to 55%; with two steps by 17 to 58%, for 2% of the fp32
+// step at B4 T1000 d768 H12 k125: 208 against 212.6 us).
+constexpr int kSplitAcc = 4;
 template <class Op>
 constexpr int split_smem() {
     return 1024 + split_stages<Op>() * (Op::kPA + Op::kPB) * kSplitPlane + kSplitOut + 256;
+}
+
+// Two fp32 values rounded to bf16, x in the low half; beyond the bf16 range, infinities
+// included, the largest bf16 value of that sign (NaN stays NaN).
+__device__ __forceinline__ uint32_t bf16x2_sat(float x, float y) {
+    uint32_t r;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
+    return r;
 }
 
 // Eight fp32 values as three planes of eight bf16 (16 bytes each).
 __device__ __forceinline__ void split3(const float4 &x, const float4 &y, uint4 (&pl)[3]) {
     const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
     uint32_t w[3][4];
+    auto lo = [](uint32_t u) { return __uint_as_float(u << 16); };
+    auto hi = [](uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); };
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const float a = v[2 * e], b = v[2 * e + 1];
-        const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-        const float ra = a - __uint_as_float(ua & 0xFFFF0000u);
-        const float rb = b - __uint_as_float(ub & 0xFFFF0000u);
-        const uint32_t va = __float_as_uint(ra), vb = __float_as_uint(rb);
-        const float sa = ra - __uint_as_float(va & 0xFFFF0000u);
-        const float sb = rb - __uint_as_float(vb & 0xFFFF0000u);
-        w[0][e] = __byte_perm(ua, ub, 0x7632);
-        w[1][e] = __byte_perm(va, vb, 0x7632);
-        w[2][e] = __byte_perm(__float_as_uint(sa), __float_as_uint(sb), 0x7632);
+        w[0][e] = bf16x2_sat(a, b);
+        const float ra = a - lo(w[0][e]), rb = b - hi(w[0][e]);
+        w[1][e] = bf16x2_sat(ra, rb);
+        // what is left has at most eight bits: the upper half of its fp32 form
+        w[2][e] = __byte_perm(__float_as_uint(ra - lo(w[1][e])), __float_as_uint(rb - hi(w[1][e])),
+                              0x7632);
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) pl[i] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
     constexpr bool kF32 = split_f32<Op>();
     constexpr int S = split_stages<Op>();
     constexpr int kStage = (Op::kPA + Op::kPB) * kSplitPlane;
-    constexpr int DR = split_drain<Op>(), NA = kSplitAcc;
+    constexpr int NA = kSplitAcc;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -375,52 +381,47 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
         // ----------------------------------------------------- MMA issuer
         if (elect_one()) {
             const uint32_t idesc = idesc_bf16(128, sa.bn, Op::kAMN, Op::kBMN);
-            int n = 0, c = 0;   // K blocks and accumulators so far
+            int n = 0;   // K blocks so far
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < sa.tiles; tile += step) {
                 const SplitTile tl(sa, tile);
                 for (int it = 0; it < tl.nkb; ++it, ++n) {
                     const int s = n % S;
-                    ok = mbar_wait(smem_u32(&full[s]), (n / S) & 1);
+                    ok = mbar_wait(smem_u32(&full[s]), (n / S) & 1) &&
+                         mbar_wait(smem_u32(&acce[n % NA]), ((n / NA) & 1) ^ 1);
                     if (!ok || *(volatile int *)s_abort) {
                         give_up();
                         ok = false;
                         break;
                     }
+                    tc_fence_after();
                     const uint32_t a = smem_u32(ring + s * kStage), b = a + Op::kPA * kSplitPlane;
                     const int left = op.K - (tl.kb0 + it) * 64;
                     const int steps = left >= 64 ? 4 : (left + 15) / 16;
-                    for (int st0 = 0; ok && st0 < steps; st0 += DR, ++c) {
-                        ok = mbar_wait(smem_u32(&acce[c % NA]), ((c / NA) & 1) ^ 1);
-                        if (!ok) break;
-                        tc_fence_after();
-                        uint32_t acc = 0u;
-                        auto product = [&](int i, int j) {
-                            for (int st = st0; st < min(steps, st0 + DR); ++st) {
-                                const uint32_t ai = a + i * kSplitPlane, bj = b + j * kSplitPlane;
-                                const uint64_t ad = Op::kAMN ? smem_desc_sw128(ai + st * 2048, 8192, 1024)
-                                                             : smem_desc_sw128(ai + st * 32, 16, 1024);
-                                const uint64_t bd = Op::kBMN ? smem_desc_sw128(bj + st * 2048, 8192, 1024)
-                                                             : smem_desc_sw128(bj + st * 32, 16, 1024);
-                                mma_bf16(tmem + 128 * (c % NA), ad, bd, idesc, acc);
-                                acc = 1u;
-                            }
-                        };
-                        // small products first
-                        if constexpr (kF32) {
-                            product(2, 0);
-                            product(0, 2);
-                            product(1, 1);
+                    uint32_t acc = 0u;
+                    auto product = [&](int i, int j) {
+#pragma unroll   // (left rolled, that fp32 step takes 211 us)
+                        for (int st = 0; st < 4; ++st) {
+                            if (st >= steps) break;
+                            const uint32_t ai = a + i * kSplitPlane, bj = b + j * kSplitPlane;
+                            const uint64_t ad = Op::kAMN ? smem_desc_sw128(ai + st * 2048, 8192, 1024)
+                                                         : smem_desc_sw128(ai + st * 32, 16, 1024);
+                            const uint64_t bd = Op::kBMN ? smem_desc_sw128(bj + st * 2048, 8192, 1024)
+                                                         : smem_desc_sw128(bj + st * 32, 16, 1024);
+                            mma_bf16(tmem + 128 * (n % NA), ad, bd, idesc, acc);
+                            acc = 1u;
                         }
-                        if constexpr (Op::kPA > 1) product(1, 0);
-                        if constexpr (Op::kPB > 1) product(0, 1);
-                        product(0, 0);
-                        mma_commit(smem_u32(&accf[c % NA]));
+                    };
+                    // small products first
+                    if constexpr (kF32) {
+                        product(2, 0);
+                        product(0, 2);
+                        product(1, 1);
                     }
-                    if (!ok) {
-                        give_up();
-                        break;
-                    }
+                    if constexpr (Op::kPA > 1) product(1, 0);
+                    if constexpr (Op::kPB > 1) product(0, 1);
+                    product(0, 0);
+                    mma_commit(smem_u32(&accf[n % NA]));
                     mma_commit(smem_u32(&empty[s]));
                 }
             }
@@ -431,16 +432,14 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
         const int q = warp & 3, hf = warp >> 2;
         const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + 64 * hf;
         uint8_t *xb = outs + warp * 4096;
-        int c = 0;
+        int c = 0;   // K blocks so far
         bool ok = true;
         for (int tile = blockIdx.x; ok && tile < sa.tiles; tile += step) {
             const SplitTile tl(sa, tile);
             float v[64];
 #pragma unroll
             for (int j = 0; j < 64; ++j) v[j] = 0.f;
-            const int k16 = (min(op.K, (tl.kb0 + tl.nkb) * 64) - tl.kb0 * 64 + 15) / 16;
-            const int chunks = (k16 + DR - 1) / DR;   // (<= 0 for a split with no K blocks)
-            for (int u = 0; u < chunks; ++u, ++c) {
+            for (int u = 0; u < tl.nkb; ++u, ++c) {
                 ok = mbar_wait(smem_u32(&accf[c % NA]), (c / NA) & 1);
                 // warp-uniform: the TMEM loads below are warp-collective
                 if (__any_sync(0xffffffffu, !ok || *(volatile int *)s_abort)) {
