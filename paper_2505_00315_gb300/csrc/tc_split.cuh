@@ -16,8 +16,7 @@
 // drained into fp32 registers after every 64-wide K block, so that the tensor
 // pipe's accumulation rounding acts on short partial sums only.
 //
-// Results around an infinity, or past the fp32 range, can come out as NaN where a plain
-// product is infinite: results around a NaN are computed again with plain fp32 multiply-adds.
+// Non-finite results are those of plain products (see store_non_finite).
 //
 // One CTA (544 threads) per SM walks over 128 x bn tiles (bn <= 128) of all groups:
 //   warps 0-7    drain: TMEM -> registers (four accumulators in turn), then the
@@ -39,6 +38,8 @@
 // cycles a block, where the CUDA-core product it replaces needed 4096 at the FFMA
 // rate and ran at a tenth of that.
 #pragma once
+
+#include <cfloat>
 
 #include "launch.h"
 #include "profile.h"
@@ -137,6 +138,85 @@ struct SplitTile {
         m0 = (int)m * 128;
     }
 };
+
+// Non-finite results of a warp's 32 rows x 64 columns.  Where an operand is not finite they
+// are right: an infinity is cut into (largest, largest, infinity), p2 meets q0 only, and
+// that product comes first, so that it decides the sign (or NaN, times 0).  Where
+// both operands are finite and their product passes the fp32 range 2^8 times over, p1 q0 or p0 q1
+// does so before p0 q0, with either sign: such elements (non-finite, no non-finite
+// operand) are computed again by plain multiply-adds.  Rows and columns that are NaN throughout
+// come from a NaN operand and need no look at the operands.
+// The issuer waits meanwhile, with a limit: at most kPlainSteps steps (about 0.2 s) a tile.
+// (All results of a warp with a NaN again, each by a chain over all of K: a step of B4 T2048
+// d768 H12 k512 with one NaN in X took 44 ms instead of 0.7, and takes 1.0 now.)
+constexpr int kPlainSteps = 1 << 22;   // 64 columns of 65536 rows
+// Puts v's columns nb .. nb + w - 1 of row m right and stores them (w and the number of rows
+// are the same in all lanes).  Out of line, and on a copy of the results, so that the
+// output step around it keeps them in registers.
+template <class Op>
+__device__ __noinline__ void store_non_finite(const Op &op, int g, int sp, int m, int rows, int nb,
+                                              int w, int k0, int k1, float *v) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    if (rows <= 0) return;
+    const bool mine = lane < rows;
+    uint32_t todo[2] = {0u, 0u}, nan[2] = {0u, 0u};
+    for (int j = 0; j < w; ++j) {
+        const float x = mine ? v[j] : 0.f;
+        const bool is_nan = x != x;
+        const bool column = __popc(__ballot_sync(kAll, is_nan)) == rows;
+        if (is_nan) nan[j >> 5] |= 1u << (j & 31);
+        if (!column && !(fabsf(x) <= FLT_MAX)) todo[j >> 5] |= 1u << (j & 31);
+    }
+    if (__popc(nan[0]) + __popc(nan[1]) == w) todo[0] = todo[1] = 0u;
+    int steps = kPlainSteps - 3 * min(k1 - k0, kPlainSteps);
+    if (steps < 0) todo[0] = todo[1] = 0u;
+    constexpr int U = 8;   // steps whose loads are in flight at a time (past the end, the last again)
+    const int row = mine ? m : m - lane;
+    if (__any_sync(kAll, (todo[0] | todo[1]) != 0u)) {
+        const int c0 = nb + min(lane, w - 1), c1 = nb + min(lane + 32, w - 1);
+        float za = 0.f, z0 = 0.f, z1 = 0.f;   // 0 times a non-finite value is NaN
+        for (int k = k0; k < k1; k += U) {
+            float a[U], b0[U], b1[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int kk = min(k + i, k1 - 1);
+                a[i] = op.a(g, row, kk);
+                b0[i] = op.b(g, kk, c0);
+                b1[i] = op.b(g, kk, c1);
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                za = fmaf(a[i], 0.f, za);
+                z0 = fmaf(b0[i], 0.f, z0);
+                z1 = fmaf(b1[i], 0.f, z1);
+            }
+        }
+        const uint32_t bad0 = __ballot_sync(kAll, z0 != 0.f), bad1 = __ballot_sync(kAll, z1 != 0.f);
+        todo[0] = za != 0.f ? 0u : todo[0] & ~bad0;
+        todo[1] = za != 0.f ? 0u : todo[1] & ~bad1;
+    }
+    for (int j = 0; j < w; ++j) {
+        float x = v[j];
+        const bool on = todo[j >> 5] >> (j & 31) & 1u;
+        if (__any_sync(kAll, on) && (steps -= k1 - k0) >= 0) {
+            float acc = 0.f;
+            for (int k = k0; k < k1; k += U) {
+                float a[U], b[U];
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    const int kk = min(k + i, k1 - 1);
+                    a[i] = op.a(g, row, kk);
+                    b[i] = k + i < k1 ? op.b(g, kk, nb + j) : 0.f;   // (a is finite)
+                }
+#pragma unroll
+                for (int i = 0; i < U; ++i) acc = fmaf(a[i], b[i], acc);
+            }
+            if (on) x = acc;
+        }
+        if (mine) op.store(g, m, nb + j, x, sp);
+    }
+}
 
 template <class Op>
 __global__ void __launch_bounds__(kSplitThreads, 1)
@@ -464,21 +544,17 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
             if (tile + step >= sa.tiles) pdl_trigger();
             const int nb = tl.n0 + 64 * hf, n_end = min(op.N, tl.n0 + sa.bn);
             const int m = tl.m0 + q * 32 + lane;
-            if constexpr (kF32) {
-                bool nan = false;
+            if constexpr (Op::kPA + Op::kPB > 2) {
+                bool bad = false;
 #pragma unroll
-                for (int j = 0; j < 64; ++j) nan = nan || v[j] != v[j];
-                // from a non-finite input (or a sum past the range): the tile rows of
-                // this warp by plain multiply-adds instead
-                if (__any_sync(0xffffffffu, nan)) {
-                    const int k_end = min(op.K, (tl.kb0 + tl.nkb) * 64);
-                    if (m < op.M)
-                        for (int n = nb; n < min(n_end, nb + 64); ++n) {
-                            float acc = 0.f;
-                            for (int k = tl.kb0 * 64; k < k_end; ++k)
-                                acc = fmaf(op.a(tl.g, m, k), op.b(tl.g, k, n), acc);
-                            op.store(tl.g, m, n, acc, tl.sp);
-                        }
+                for (int j = 0; j < 64; ++j) bad = bad || !(fabsf(v[j]) <= FLT_MAX);
+                if (__any_sync(0xffffffffu, bad)) {
+                    float x[64];
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) x[j] = v[j];
+                    store_non_finite(op, tl.g, tl.sp, m, min(32, op.M - (tl.m0 + q * 32)), nb,
+                                     min(64, n_end - nb), tl.kb0 * 64,
+                                     min(op.K, (tl.kb0 + tl.nkb) * 64), x);
                     continue;
                 }
             }
