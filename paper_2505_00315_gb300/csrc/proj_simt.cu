@@ -263,6 +263,8 @@ struct WBwdOp {
             put1(dst(g, c, n), v, sp >= 0);
         else if (n == 3 * hp)
             put1(dWr + (size_t)c * H + g, v, sp >= 0);
+        else if (v != 0.f)   // dlogit's second column, after the first by the same thread
+            atomicAdd(dWr + (size_t)c * H + g, v);
     }
     __device__ void store4(int g, int c, int n, const float4 &v, int sp) const {
         if (n < 3 * hp)
@@ -307,15 +309,15 @@ __global__ void out_bwd_rows_kernel(float *G, const float *A,
         if constexpr (std::is_same<TS, float>::value) {
             static_cast<float *>(dQKV)[row * 4 * hp + 3 * hp] = dl;
         } else {
-            // three bf16 parts (a non-finite value only in the first)
+            // three bf16 parts (a non-finite value only in the first), and zeros in the rest of
+            // the eight columns that the dW product loads
             bf16 *q = static_cast<bf16 *>(dQKV) + row * 8 * hp + 3 * hp;
             const bf16 h = __float2bfloat16_rn(dl);
             const float r1 = fabsf(dl) <= 3.38e38f ? dl - __bfloat162float(h) : 0.f;
             const bf16 l = __float2bfloat16_rn(r1);
-            q[0] = h;
-            q[4 * hp] = l;
-            q[1] = __float2bfloat16_rn(r1 - __bfloat162float(l));
-            q[4 * hp + 1] = __float2bfloat16_rn(0.f);
+            const __nv_bfloat162 hi = __halves2bfloat162(h, __float2bfloat16_rn(r1 - __bfloat162float(l)));
+            *reinterpret_cast<uint4 *>(q) = make_uint4(*reinterpret_cast<const uint32_t *>(&hi), 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(q + 4 * hp) = make_uint4(__bfloat16_as_ushort(l), 0u, 0u, 0u);
         }
     }
 }

@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_2505_00315_gb300 as mosa
 from paper_2505_00315_gb300 import workloads as W
-from _gpu import run_layer
+from _gpu import run_layer, to_dev
 from _util import rel_l2
 
 pytestmark = pytest.mark.gpu
@@ -122,3 +122,19 @@ def test_one_nan_does_not_slow_an_f32_layer():
     assert all(torch.isnan(got[n]).any() for n in ("dX", "dW_q", "dW_o"))
     # (not once: the CUDA-core attention has a slower branch for tiles with non-finite values)
     assert nan < 2.0 * plain, (nan, plain)
+
+
+def test_weight_gradients_do_not_hang_on_the_workspace_contents():
+    # bf16 with heads of 128: dlogit's two columns of the dW product lie beside unused ones
+    cfg = W.MosaConfig("stale_workspace", B=2, T=150, d=264, H=20, hp=128, k=66, dtype="bf16", seed=87)
+    x = W.make_inputs(cfg)
+    X, Wr, Wq, Wk, Wv, Wo, dY = (to_dev(x[n], "bf16")
+                                 for n in ("X", "Wr", "Wq", "Wk", "Wv", "Wo", "dY"))
+    got = []
+    for fill in (0, 255):
+        ws = mosa.alloc_workspace(mosa.make_shape(X, Wq, cfg.k)).fill_(fill)
+        _, I, rs, _, ws = mosa.mosa_forward(X, Wr, Wq, Wk, Wv, Wo, cfg.k, workspace=ws)
+        got.append(mosa.mosa_backward(X, Wr, Wq, Wk, Wv, Wo, I, rs, dY, ws))
+    torch.cuda.synchronize()
+    for n in ("dW_r", "dW_q", "dW_k", "dW_v", "dW_o"):
+        assert torch.equal(got[0][n], got[1][n]), n
