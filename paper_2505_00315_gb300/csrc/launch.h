@@ -12,47 +12,25 @@
 
 namespace mosa {
 
-// Launches `kernel` with programmatic stream serialization when `early` (it
-// may begin while the preceding kernel on the stream finishes; the kernel
-// itself waits with griddepcontrol.wait before reading that kernel's results).
-// A kernel that shares the GPU with another stream's kernel is launched late
-// instead: waiting early, its CTAs would hold SMs the other kernel needs.
-// MOSA_PDL=0 launches every kernel plainly.
-// priority (when not 0): the launch's scheduling priority, lower is sooner.
-template <class... KArgs, class... Args>
-inline cudaError_t launch_ex(bool early, int priority, void (*kernel)(KArgs...), dim3 grid,
-                             dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
+// Launches `kernel` with programmatic stream serialization (it may begin while the
+// preceding kernel on the stream finishes; the kernel itself waits with
+// griddepcontrol.wait before reading that kernel's results), at the stream's
+// priority.  MOSA_PDL=0 launches every kernel plainly.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t s, Args &&...args) {
     const char *v = std::getenv("MOSA_PDL");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    if (early && (v == nullptr || v[0] != '0')) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
-    if (priority != 0) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributePriority;
-        attr[cfg.numAttrs++].val.priority = priority;
-    }
+    cfg.numAttrs = v != nullptr && v[0] == '0' ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t s, Args &&...args) {
-    return launch_ex(true, 0, kernel, grid, block, smem, s, std::forward<Args>(args)...);
-}
-// As launch_pdl, ahead of the side stream's copies and zeroing: the kernels that
-// follow TopK on the caller's stream (the greatest priority of the device).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_ahead(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                cudaStream_t s, Args &&...args) {
-    int least = 0, greatest = 0;
-    (void)cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    return launch_ex(true, greatest, kernel, grid, block, smem, s, std::forward<Args>(args)...);
 }
 
 // Raises `kernel`'s dynamic shared-memory limit to `bytes` on the current

@@ -140,9 +140,9 @@ constexpr int kMaxPrio = 8;   // stream priorities 0, -1, ..
 std::mutex g_res_mu;
 DevResources g_res[kMaxDev][kMaxPrio];
 
-// Priority of the caller's stream as an index 0 .. kMaxPrio - 1 (0: the default).
-// Layer graphs run by the priorities of their nodes (cudaGraphInstantiateFlagUseNodePriority),
-// so the internal streams a call is captured on take the caller's.
+// Priority of the caller's stream as an index 0 .. kMaxPrio - 1 (0: the default): the
+// internal streams take the caller's.  (A layer graph runs at that of the stream
+// it is launched on.)
 int priority_index(cudaStream_t s) {
     int prio = 0;
     if (cudaStreamGetPriority(s, &prio) != cudaSuccess) return 0;
@@ -554,7 +554,7 @@ bool side_by_side(Hybrid *h, HybridSpace *sp) {
 // graph on the caller's stream.  MOSA_GRAPHS=0 turns this off.
 
 struct GraphKey {
-    int op, device, tc, prio;
+    int op, device, tc;
     uint32_t mask;
     mosa_shape shape;
     int extra[2];  // hybrid calls: dense heads, window
@@ -579,7 +579,7 @@ struct GraphEntry {
 constexpr size_t kMaxGraphs = 128;
 std::mutex g_graph_mu;
 std::unordered_map<GraphKey, GraphEntry *, GraphKeyHash> g_graphs;
-cudaStream_t g_capture_stream[kMaxDev][kMaxPrio] = {};
+cudaStream_t g_capture_stream[kMaxDev] = {};
 
 bool graphs_enabled() {
     const char *v = std::getenv("MOSA_GRAPHS");
@@ -591,13 +591,12 @@ int path_bits(const Dims &dm) {
            (use_headsum_out(dm) ? 8 : 0) | (use_headsum_dx(dm) ? 16 : 0) | (use_split() ? 32 : 0);
 }
 
-GraphKey make_key(int op, int prio, const Dims &dm, const mosa_shape *shape,
+GraphKey make_key(int op, const Dims &dm, const mosa_shape *shape,
                   std::initializer_list<const void *> ptrs, const Dims *dense = nullptr,
                   int extra0 = 0, int extra1 = 0) {
     GraphKey k;
     std::memset(&k, 0, sizeof(k));
     k.op = op;
-    k.prio = prio;
     cudaGetDevice(&k.device);
     k.tc = path_bits(dm) | (dense ? path_bits(*dense) << 6 : 0);
     k.mask = profile_mask();
@@ -620,9 +619,8 @@ mosa_status run_graphed(const GraphKey &key, cudaStream_t user, Enqueue &&enqueu
     GraphEntry *e = it == g_graphs.end() ? nullptr : it->second;
     if (e == nullptr) {
         if (g_graphs.size() >= kMaxGraphs) return enqueue(user);
-        cudaStream_t &cs = g_capture_stream[key.device][key.prio];
-        if (cs == nullptr &&
-            cudaStreamCreateWithPriority(&cs, cudaStreamNonBlocking, -key.prio) != cudaSuccess) {
+        cudaStream_t &cs = g_capture_stream[key.device];
+        if (cs == nullptr && cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
             cs = nullptr;
             return enqueue(user);
         }
@@ -635,8 +633,7 @@ mosa_status run_graphed(const GraphKey &key, cudaStream_t user, Enqueue &&enqueu
             if (cudaStreamEndCapture(cs, &g) != cudaSuccess) st = MOSA_ERR_CUDA;
         }
         capture_into(nullptr);
-        if (st == MOSA_OK && g != nullptr &&
-            cudaGraphInstantiate(&e->exec, g, cudaGraphInstantiateFlagUseNodePriority) != cudaSuccess)
+        if (st == MOSA_OK && g != nullptr && cudaGraphInstantiate(&e->exec, g, 0) != cudaSuccess)
             st = MOSA_ERR_CUDA;
         if (g != nullptr) cudaGraphDestroy(g);
         if (st != MOSA_OK) {
@@ -705,7 +702,7 @@ mosa_status mosa_forward(const mosa_shape *shape, const void *X, const void *W_r
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         return forward_routed(dm, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf, sv, s, res);
     };
-    const GraphKey key = make_key(0, prio, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, r_full,
+    const GraphKey key = make_key(0, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, r_full,
                                                  workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
@@ -725,7 +722,7 @@ mosa_status mosa_forward_with_indices(const mosa_shape *shape, const void *X, co
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         return forward_given(dm, X, W_q, W_k, W_v, W_o, I, r_sel, Y, sv, s, res);
     };
-    const GraphKey key = make_key(1, prio, dm, shape, {X, W_q, W_k, W_v, W_o, I, r_sel, Y, workspace});
+    const GraphKey key = make_key(1, dm, shape, {X, W_q, W_k, W_v, W_o, I, r_sel, Y, workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
 
@@ -748,7 +745,7 @@ mosa_status mosa_backward(const mosa_shape *shape, const void *X, const void *W_
         return backward_all(dm, X, W_r, W_q, W_k, W_v, W_o, dY, dX, dW_r, dW_q, dW_k, dW_v, dW_o,
                             sv, s, res);
     };
-    const GraphKey key = make_key(2, prio, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, I, r_sel, dY, dX,
+    const GraphKey key = make_key(2, dm, shape, {X, W_r, W_q, W_k, W_v, W_o, I, r_sel, dY, dX,
                                                  dW_r, dW_q, dW_k, dW_v, dW_o, workspace});
     return run_graphed(key, (cudaStream_t)stream, enqueue);
 }
@@ -797,7 +794,7 @@ mosa_status mosa_hybrid_forward(const mosa_hybrid_shape *shape, const void *X, c
         MOSA_TRY(link(res->dense, s, res->dense_done));
         return MOSA_OK;
     };
-    const GraphKey key = make_key(3, prio, h.sparse, &shape->sparse,
+    const GraphKey key = make_key(3, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, Y, I, r_sel,
                                    r_full, workspace},
                                   h.has_dense ? &h.dense : nullptr, shape->H_dense, shape->window);
@@ -848,7 +845,7 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
         MOSA_TRY(link(ds, s, res->dense_done));
         return MOSA_OK;
     };
-    const GraphKey key = make_key(4, prio, h.sparse, &shape->sparse,
+    const GraphKey key = make_key(4, h.sparse, &shape->sparse,
                                   {X, W_r, W_q, W_k, W_v, W_o, D_q, D_k, D_v, D_o, I, r_sel, dY,
                                    dX, dW_r, dW_q, dW_k, dW_v, dW_o, dD_q, dD_k, dD_v, dD_o,
                                    workspace},

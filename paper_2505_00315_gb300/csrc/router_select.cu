@@ -736,9 +736,9 @@ cudaError_t launch_select(int rows, int T, int k, const float *scores, int32_t *
                           bool first_token) {
     if (rows <= 0) return cudaSuccess;
     if (T > 16 * kSelThreads) {
-        const cudaError_t e = launch_ahead(topk_long_kernel, dim3(rows), dim3(kSelThreads), 0, stream,
-                                           scores, T, k, I, rsel, B, H, gidx, rsel_hm,
-                                           first_token ? 1 : 0, active_span());
+        const cudaError_t e = launch_pdl(topk_long_kernel, dim3(rows), dim3(kSelThreads), 0, stream,
+                                         scores, T, k, I, rsel, B, H, gidx, rsel_hm,
+                                         first_token ? 1 : 0, active_span());
         note_launches(1);
         return e;
     }
@@ -748,8 +748,8 @@ cudaError_t launch_select(int rows, int T, int k, const float *scores, int32_t *
     auto threads = [&]() { return ((T + 4 * V - 1) / (4 * V) + 31) / 32 * 32; };
     while (V < kSelMaxVec && (threads() > kSelThreads || (long long)rows * threads() > 152 * 1024)) V *= 2;
     auto kern = V == 1 ? topk_select_kernel<1> : V == 2 ? topk_select_kernel<2> : topk_select_kernel<4>;
-    const cudaError_t e = launch_ahead(kern, dim3(rows), dim3(threads()), 0, stream, scores, T, k, I,
-                                       rsel, B, H, gidx, rsel_hm, first_token ? 1 : 0, active_span());
+    const cudaError_t e = launch_pdl(kern, dim3(rows), dim3(threads()), 0, stream, scores, T, k, I,
+                                     rsel, B, H, gidx, rsel_hm, first_token ? 1 : 0, active_span());
     note_launches(1);
     return e;
 }

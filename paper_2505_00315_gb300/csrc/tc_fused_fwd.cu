@@ -493,7 +493,7 @@ cudaError_t tc_fused_forward(const Dims &dm, const void *X, const void *Wq, cons
     const int tiles = (dm.B + p.U - 1) / p.U * dm.H;
     const int parts = std::max(1, std::min((dm.d + kChunk - 1) / kChunk, 152 / tiles));
     const dim3 grid((dm.B + p.U - 1) / p.U, dm.H, parts);
-    cudaError_t e = launch_ahead(fused_fwd_kernel, grid, dim3(kThreads), kSmem, s, p);
+    cudaError_t e = launch_pdl(fused_fwd_kernel, grid, dim3(kThreads), kSmem, s, p);
     note_launches(1);
     return e;
 }

@@ -845,9 +845,7 @@ cudaError_t launch_kind(const TcParams &p, dim3 grid, cudaStream_t s) {
     if (p.wait_ns == 0) return cudaErrorInvalidValue;  // every launcher sets a wait limit
     const cudaError_t attr = allow_smem((const void *)tc_gemm_kernel<KIND>, smem);
     if (attr != cudaSuccess) return attr;
-    cudaError_t e = KIND == kQKV
-                        ? launch_ahead(tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p)
-                        : launch_pdl(tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p);
+    cudaError_t e = launch_pdl(tc_gemm_kernel<KIND>, grid, dim3(kThreads), smem, s, p);
     note_launches(1);
     return e;
 }
@@ -922,11 +920,14 @@ bool tc_router(const Dims &dm, const void *X, const void *Wr, int wr_cols, float
 // Side-stream work of the forward: the fp16 copies (bf16x8_to_f16x8; a value
 // beyond the fp16 range sets kStatusRange) and zeroing.  Each CTA of 256
 // threads handles one 16-byte unit per thread and ends, so that TopK and the
-// kernel after it, launched ahead of these in priority, get an SM as soon as a few
+// kernel after it get an SM as soon as a few
 // of them have ended: with grid-stride CTAs over whole copies the kernel after TopK
 // waited until the copies were through (16 us at B16 T1024 d1024 H64 k64, whose
 // step went from 375 to 365 us; B2 T8192 d1024 H32 k256 168.5 -> 164; four
-// units per thread in flight slowed TopK: 371 and 166).
+// units per thread in flight slowed TopK: 371 and 166).  A launch priority above these for
+// TopK and the kernel after it gains nothing more (B16 T1024 d1024 H64 k64 364.2 us with it, 363.3
+// without, B2 T8192 157.3 and 158.4, B4 T4096 d1024 H8 k2048 359.8 and 362.4), and would
+// put them ahead of the caller's other streams.
 constexpr int kSideCta = 256;   // units per CTA
 
 struct F16Copies {
