@@ -772,18 +772,18 @@ mosa_status mosa_hybrid_forward(const mosa_hybrid_shape *shape, const void *X, c
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sp.sparse.r_full;
     const int prio = priority_index((cudaStream_t)stream);
-    DevResources *res = dev_resources(prio);
-    if (res == nullptr) return MOSA_ERR_CUDA;
-    const bool both = side_by_side(&h, &sp);
+    // (both head groups have the same dtype and head size, so also the same path)
+    DevResources *res = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
+    const bool both = res != nullptr && side_by_side(&h, &sp);
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         if (both) MOSA_TRY(cudaMemsetAsync(sp.sparse.status, 0, sizeof(uint32_t), s));
         if (both) MOSA_TRY(cudaEventRecord(res->fork, s));
         mosa_status e = forward_routed(h.sparse, X, W_r, W_q, W_k, W_v, W_o, Y, I, r_sel, rf,
-                                       sp.sparse, s, use_tc(h.sparse) ? res : nullptr);
+                                       sp.sparse, s, res);
         if (e != MOSA_OK || !h.has_dense) return e;
         if (!both)
             return forward_given(h.dense, X, D_q, D_k, D_v, D_o, nullptr, nullptr, Y, sp.dense, s,
-                                 use_tc(h.dense) ? res : nullptr);
+                                 res);
         MOSA_TRY(cudaEventRecord(res->heads_done, s));
         MOSA_TRY(cudaStreamWaitEvent(res->dense, res->fork, 0));
         DevResources d = res->dense_set();
@@ -820,14 +820,13 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     const int prio = priority_index((cudaStream_t)stream);
-    DevResources *res = dev_resources(prio);
-    if (res == nullptr) return MOSA_ERR_CUDA;
-    const bool both = side_by_side(&h, &sp);
+    // (both head groups have the same dtype and head size, so also the same path)
+    DevResources *res = use_tc(h.sparse) ? dev_resources(prio) : nullptr;
+    const bool both = res != nullptr && side_by_side(&h, &sp);
     auto enqueue = [&](cudaStream_t s) -> mosa_status {
         if (both) MOSA_TRY(cudaEventRecord(res->fork, s));
         mosa_status e = backward_all(h.sparse, X, W_r, W_q, W_k, W_v, W_o, dY, dX, dW_r, dW_q,
-                                     dW_k, dW_v, dW_o, sp.sparse, s,
-                                     use_tc(h.sparse) ? res : nullptr);
+                                     dW_k, dW_v, dW_o, sp.sparse, s, res);
         if (e != MOSA_OK || !h.has_dense) return e;
         cudaStream_t ds = both ? res->dense : s;
         if (both) {
@@ -837,7 +836,7 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
         MOSA_TRY(cudaMemsetAsync(sp.zero_wr, 0, sp.zero_wr_bytes, ds));
         if (!both)
             return backward_all(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q,
-                                dD_k, dD_v, dD_o, sp.dense, s, use_tc(h.dense) ? res : nullptr);
+                                dD_k, dD_v, dD_o, sp.dense, s, res);
         DevResources d = res->dense_set();
         e = backward_tc(h.dense, X, sp.zero_wr, D_q, D_k, D_v, D_o, dY, dX, sp.dwr, dD_q, dD_k, dD_v,
                         dD_o, sp.dense, ds, d, res->heads_done);
