@@ -125,6 +125,8 @@ bool tc_supported(const Dims &dm);
 // value: the projections then run on the CUDA cores for every shape (else on the tensor
 // cores, those of fp32 storage and other head sizes through bf16 planes).
 bool use_split();
+// fp32 values of scratch that the weight gradients' reduction splits need (Saved::wpart).
+size_t split_part_floats(const Dims &dm);
 // True when the tensor-core kernels serve this shape (false also when the
 // environment variable MOSA_FORCE_SIMT is set to a non-zero value).
 bool use_tc(const Dims &dm);

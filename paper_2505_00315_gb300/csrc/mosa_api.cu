@@ -81,6 +81,7 @@ size_t carve(const Dims &dm, char *base, Saved *sv) {
         s.AR16 = take((size_t)2 * R * dm.hp);
         s.pos = (int32_t *)take(sizeof(int32_t) * (size_t)dm.H * dm.B * dm.T);
     }
+    if (!dm.bf16 || dm.hp != 64) s.wpart = (float *)take(sizeof(float) * split_part_floats(dm));
     if (sv) *sv = s;
     return off;
 }

@@ -54,19 +54,20 @@ __device__ __forceinline__ void st_inter4(void *p, size_t row, int cols, int c, 
     }
 }
 
-// The result of one reduction split: four columns, or one value.
-__device__ __forceinline__ void put4(float *dst, const float4 &v, bool add) {
-    if (add)
-        tc::red_add_v4(dst, v.x, v.y, v.z, v.w);
-    else
-        *reinterpret_cast<float4 *>(dst) = v;
-}
-__device__ __forceinline__ void put1(float *dst, float v, bool add) {
-    if (add)
-        atomicAdd(dst, v);
-    else
-        *dst = v;
-}
+// Weight gradients in reduction splits: split 0 (or the only one) goes to the output,
+// split j to the j-th array of partial sums, laid out as the outputs one after the
+// other; sum_splits_kernel adds them up, so that each gradient stays one fixed sum.
+// (Added to the outputs as they came, more than two splits gave other last bits from
+// call to call, and their zeroing took longer than this: fp32 steps of B4 T1000 d768 H12 k125
+// 208.7 -> 202.4 us, B2 T2048 d256 H4 k512 240 -> 226.)
+struct Parts {
+    float *part;
+    size_t stride;   // of one split's partial sums
+    // where split sp puts element i of the output that starts `before` elements into the layout
+    __device__ __forceinline__ float *at(float *out, size_t before, size_t i, int sp) const {
+        return sp <= 0 ? out + i : part + (size_t)(sp - 1) * stride + before + i;
+    }
+};
 
 template <class T>
 struct QkvOp {
@@ -175,6 +176,7 @@ struct OutBwdWOp {
     const T *AR;
     const int32_t *gidx;
     float *dWo;
+    Parts parts;
     int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
     __device__ int a_row(int g, int m) const { return gidx[(size_t)g * K + m]; }
     __device__ const T *b_ptr(int g, int m, int p) const {
@@ -183,7 +185,7 @@ struct OutBwdWOp {
     __device__ float a(int g, int c, int m) const { return to_f32(A[(size_t)a_row(g, m) * M + c]); }
     __device__ float b(int g, int m, int p) const { return Inter<TS>::ld(AR, (size_t)g * K + m, N, p); }
     __device__ void store(int g, int c, int p, float v, int sp) const {
-        put1(dWo + ((size_t)g * N + p) * M + c, v, sp >= 0);
+        *parts.at(dWo, 0, ((size_t)g * N + p) * M + c, sp) = v;
     }
     __device__ void store4(int, int, int, const float4 &, int) const {}
 };
@@ -243,6 +245,8 @@ struct WBwdOp {
     const float *dlogit;
     const int32_t *gidx;
     float *dWq, *dWk, *dWv, *dWr;
+    Parts parts;
+    size_t n1;   // elements of dWq (and dWk, dWv)
     int lda = 0, a_lo = 0, ldb = 0, b_lo = 0;
     __device__ int a_row(int g, int m) const { return gidx[(size_t)g * K + m]; }
     __device__ const T *b_ptr(int g, int m, int n) const {
@@ -254,23 +258,24 @@ struct WBwdOp {
         if (n > 3 * hp) return 0.f;   // (dlogit's rounding remainder, in its fp32 value already)
         return n < 3 * hp ? Inter<TS>::ld(dQKV, row, 4 * hp, n) : dlogit[row];
     }
-    __device__ float *dst(int g, int c, int n) const {
+    __device__ float *dst(int g, int c, int n, int sp) const {
+        if (n >= 3 * hp) return parts.at(dWr, 3 * n1, (size_t)c * H + g, sp);
         const int w = n >> lg, p = n & (hp - 1);
-        return (w == 0 ? dWq : (w == 1 ? dWk : dWv)) + ((size_t)g * M + c) * hp + p;
+        return parts.at(w == 0 ? dWq : (w == 1 ? dWk : dWv), w * n1, ((size_t)g * M + c) * hp + p, sp);
     }
     __device__ void store(int g, int c, int n, float v, int sp) const {
-        if (n < 3 * hp)
-            put1(dst(g, c, n), v, sp >= 0);
-        else if (n == 3 * hp)
-            put1(dWr + (size_t)c * H + g, v, sp >= 0);
+        float *p = dst(g, c, n, sp);
+        if (n <= 3 * hp)
+            *p = v;
         else if (v != 0.f)   // dlogit's second column, after the first by the same thread
-            atomicAdd(dWr + (size_t)c * H + g, v);
+            *p += v;
     }
     __device__ void store4(int g, int c, int n, const float4 &v, int sp) const {
+        float *p = dst(g, c, n, sp);
         if (n < 3 * hp)
-            put4(dst(g, c, n), v, sp >= 0);
+            *reinterpret_cast<float4 *>(p) = v;
         else
-            put1(dWr + (size_t)c * H + g, kExtra == 2 ? v.x + v.y : v.x, sp >= 0);
+            *p = kExtra == 2 ? v.x + v.y : v.x;
     }
 };
 
@@ -322,6 +327,24 @@ __global__ void out_bwd_rows_kernel(float *G, const float *A,
     }
 }
 
+// Adds the partial sums of `parts` splits, each n[0] + .. + n[3] values, to out[0] .. out[3].
+struct SumSplits {
+    float *out[4];
+    size_t n[4];
+};
+__global__ void sum_splits_kernel(const SumSplits o, const float *part, size_t stride, int parts) {
+    tc::pdl_wait();
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= stride) return;
+    int a = 0;
+    size_t at = i;
+    while (at >= o.n[a]) at -= o.n[a++];
+    float v = o.out[a][at];
+#pragma unroll 8
+    for (int j = 0; j < parts; ++j) v += part[(size_t)j * stride + i];
+    o.out[a][at] = v;
+}
+
 bool aligned16(std::initializer_list<const void *> ps) {
     uintptr_t u = 0;
     for (const void *p : ps) u |= reinterpret_cast<uintptr_t>(p);
@@ -342,6 +365,23 @@ int log2_of(int hp) {   // 16, 32, 64 or 128
 
 cudaError_t zero(float *p, size_t n, cudaStream_t s) {
     return cudaMemsetAsync(p, 0, sizeof(float) * n, s);
+}
+
+// Reduction splits of dW_o and of dW_q|dW_k|dW_v|dW_r, and the values of one split's
+// partial sums.
+int dwo_splits(const Dims &dm) { return split_count(dm.d, dm.hp, dm.B * dm.k, dm.H); }
+int dw_splits(const Dims &dm) {
+    return split_count(dm.d, 3 * dm.hp + (dm.bf16 ? 2 : 1), dm.B * dm.k, dm.H);
+}
+size_t dwo_floats(const Dims &dm) { return (size_t)dm.H * dm.hp * dm.d; }
+size_t dw_floats(const Dims &dm) { return 3 * dwo_floats(dm) + (size_t)dm.d * dm.H; }
+
+cudaError_t sum_splits(const SumSplits &o, const Saved &sv, size_t stride, int splits, cudaStream_t s) {
+    if (splits <= 1) return cudaSuccess;
+    const cudaError_t e = launch_pdl(sum_splits_kernel, dim3((unsigned)((stride + 255) / 256)), dim3(256),
+                                     0, s, o, (const float *)sv.wpart, stride, splits - 1);
+    note_launches(1);
+    return e;
 }
 
 template <class T>
@@ -368,7 +408,7 @@ cudaError_t out_t(const Dims &dm, const void *Wo, const Saved &sv, float *Y, cud
 }
 
 // G has one column tile per 128 rows: as many reduction splits as the 152 SMs have
-// room for, each of at least three K blocks and none of them empty.
+// room for, each of at least three K blocks (the last may find fewer left, none is empty).
 // fp32 at B4 T1000 d768 H12 k125, 48 tiles: 28 -> 15 us on 144 CTAs, its step 225 -> 210.
 // bf16 storage, whose K blocks are only copied, keeps one: at B4 T1024 d1024 H16 h'=128
 // k128, 64 tiles, two splits took 17 -> 13 us here and the step 285.6 -> 286.5.
@@ -398,13 +438,14 @@ cudaError_t out_bwd_t(const Dims &dm, const void *Wo, const void *dY, const Save
                    (const float *)sv.rsel, sv.dA, sv.Dd, sv.dlogit, sv.dQKV, rows, dm.hp, gsplits);
     note_launches(1);
     if (e != cudaSuccess) return e;
-    const int splits = split ? split_count(dm.d, dm.hp, Mtok, dm.H) : 1;
-    if (splits > 1 && (e = zero(dWo, (size_t)dm.H * dm.hp * dm.d, s)) != cudaSuccess) return e;
-    OutBwdWOp<T> w{dm.d, dm.hp, Mtok, (const T *)dY, (const T *)sv.AR, sv.gidx, dWo};
+    const int splits = split ? dwo_splits(dm) : 1;
+    const size_t n = dwo_floats(dm);
+    OutBwdWOp<T> w{dm.d, dm.hp, Mtok, (const T *)dY, (const T *)sv.AR, sv.gidx, dWo, {sv.wpart, n}};
     w.lda = dm.d;
     w.ldb = inter_ld<T>(dm.hp);
     w.b_lo = dm.hp;
-    return product(w, dm.H, splits, split, sv, s);
+    if ((e = product(w, dm.H, splits, split, sv, s)) != cudaSuccess) return e;
+    return sum_splits({{dWo}, {n}}, sv, n, splits, s);
 }
 
 template <class T>
@@ -427,24 +468,23 @@ cudaError_t w_bwd_t(const Dims &dm, const void *X, const Saved &sv, float *dWq, 
                     float *dWv, float *dWr, cudaStream_t s) {
     const bool split = use_split() && aligned16({X, dWq, dWk, dWv});
     const int N = 3 * dm.hp + WBwdOp<T>::kExtra, Mtok = dm.B * dm.k;
-    const int splits = split ? split_count(dm.d, N, Mtok, dm.H) : 1;
-    if (splits > 1) {
-        const size_t n = (size_t)dm.H * dm.d * dm.hp;
-        cudaError_t e;
-        if ((e = zero(dWq, n, s)) != cudaSuccess || (e = zero(dWk, n, s)) != cudaSuccess ||
-            (e = zero(dWv, n, s)) != cudaSuccess ||
-            (e = zero(dWr, (size_t)dm.d * dm.H, s)) != cudaSuccess)
-            return e;
-    }
+    const int splits = split ? dw_splits(dm) : 1;
+    const size_t n = dwo_floats(dm), stride = dw_floats(dm);
     WBwdOp<T> op{dm.d, N, Mtok, dm.hp, log2_of(dm.hp), dm.H, (const T *)X, (const T *)sv.dQKV, sv.dlogit, sv.gidx,
-                 dWq, dWk, dWv, dWr};
+                 dWq, dWk, dWv, dWr, {sv.wpart, stride}, n};
     op.lda = dm.d;
     op.ldb = inter_ld<T>(4 * dm.hp);
     op.b_lo = 4 * dm.hp;
-    return product(op, dm.H, splits, split, sv, s);
+    const cudaError_t e = product(op, dm.H, splits, split, sv, s);
+    if (e != cudaSuccess) return e;
+    return sum_splits({{dWq, dWk, dWv, dWr}, {n, n, n, (size_t)dm.d * dm.H}}, sv, stride, splits, s);
 }
 
 }  // namespace
+
+size_t split_part_floats(const Dims &dm) {
+    return std::max((dwo_splits(dm) - 1) * dwo_floats(dm), (dw_splits(dm) - 1) * dw_floats(dm));
+}
 
 bool use_split() {
     const char *f = std::getenv("MOSA_FORCE_SIMT");

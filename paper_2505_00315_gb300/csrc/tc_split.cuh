@@ -131,7 +131,7 @@ struct SplitTile {
         if (sa.splits > 1) {
             sp = (int)(t % (unsigned)sa.splits), t /= (unsigned)sa.splits;
             kb0 = sp * sa.per;
-            nkb = max(0, min(sa.nkb, kb0 + sa.per) - kb0);
+            nkb = min(sa.nkb, kb0 + sa.per) - kb0;
         }
         g = (int)t;
         n0 = (int)n * sa.bn;
@@ -279,21 +279,16 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
         auto place = [](bool mn, int row, int ch) -> uint32_t {
             return (mn ? (uint32_t)(ch >> 3) * 8192u : 0u) + row * 128 + (((ch & 7) ^ (row & 7)) << 4);
         };
-        // The K blocks of all tiles in order: (tl, it); tiles with none are skipped.
+        // The K blocks of all tiles in order: (tl, it).
         struct Walk {
             SplitTile tl;
             int tile, it;
         };
-        auto skip_empty = [&](Walk &w) {
-            while (w.tile < sa.tiles && w.it >= w.tl.nkb) {
-                w.tile += step;
-                w.it = 0;
-                if (w.tile < sa.tiles) w.tl = SplitTile(sa, w.tile);
-            }
-        };
         auto advance = [&](Walk &w) {
-            ++w.it;
-            skip_empty(w);
+            if (++w.it < w.tl.nkb) return;
+            w.tile += step;
+            w.it = 0;
+            if (w.tile < sa.tiles) w.tl = SplitTile(sa, w.tile);
         };
         // source rows of block w (-1: zeros), one per lane: a warp's chunks lie in
         // 2 (kAMN) or 4 rows of each step p, lane 2 p + i or 4 p + i holding row i's;
@@ -331,7 +326,6 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
             return first + (size_t)(kBStep * p) * op.ldb;
         };
         Walk w{SplitTile(sa, blockIdx.x), (int)blockIdx.x, 0};
-        skip_empty(w);
         int idx = -1;
         rows_of(w, idx);
         if constexpr (kF32) {
@@ -592,8 +586,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
     }
 }
 
-// Launches op over `groups` groups; splits as chosen by split_count (where it is above
-// 1 and the op's splits add up in place, the caller zeroes the output first).
+// Launches op over `groups` groups in `splits` reduction splits, none of them empty.
 template <class Op>
 inline cudaError_t launch_split_gemm(const Op &op, int groups, int splits, uint32_t *status,
                                      cudaStream_t stream) {
@@ -620,13 +613,15 @@ inline cudaError_t launch_split_gemm(const Op &op, int groups, int splits, uint3
 }
 
 // Reduction splits of a product with M x N outputs in `groups` groups over K:
-// enough tiles for the 152 SMs while each keeps at least four K blocks.
+// enough tiles for the 152 SMs while each takes at least four K blocks, of which the last
+// split may find fewer left; none is empty.
 inline int split_count(int M, int N, int K, int groups) {
-    const int tiles = (M + 127) / 128 * ((N + 127) / 128) * groups;
+    const long long tiles = (long long)((M + 127) / 128) * ((N + 127) / 128) * groups;
     const int nkb = (K + 63) / 64;
     int sp = 1;
     while (tiles * sp * 2 <= 152 && nkb / (sp * 2) >= 4) sp *= 2;
-    return sp;
+    const int per = (nkb + sp - 1) / sp;
+    return (nkb + per - 1) / per;
 }
 
 }  // namespace mosa

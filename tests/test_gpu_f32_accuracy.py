@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_2505_00315_gb300 as mosa
 from paper_2505_00315_gb300 import workloads as W
-from _gpu import run_layer, to_dev
+from _gpu import assert_close, run_layer, to_dev
 from _util import rel_l2
 
 pytestmark = pytest.mark.gpu
@@ -138,3 +138,28 @@ def test_weight_gradients_do_not_hang_on_the_workspace_contents():
     torch.cuda.synchronize()
     for n in ("dW_r", "dW_q", "dW_k", "dW_v", "dW_o"):
         assert torch.equal(got[0][n], got[1][n]), n
+
+
+# dW_o, dW_q|dW_k|dW_v and dW_r in four and more reduction splits (the second: of unequal
+# length): the same bits from call to call
+@pytest.mark.parametrize("cfg", [
+    W.MosaConfig("splits_f32", B=3, T=700, d=72, H=2, hp=32, k=345, dtype="f32", seed=88),
+    W.MosaConfig("splits_f32_uneven", B=4, T=1600, d=136, H=3, hp=64, k=520, dtype="f32", seed=89),
+    W.MosaConfig("splits_bf16", B=8, T=600, d=96, H=2, hp=32, k=300, dtype="bf16", seed=90),
+], ids=lambda c: c.name)
+def test_weight_gradients_repeat_bit_for_bit(cfg):
+    x = W.make_inputs(cfg)
+    X, Wr, Wq, Wk, Wv, Wo, dY = (to_dev(x[n], cfg.dtype)
+                                 for n in ("X", "Wr", "Wq", "Wk", "Wv", "Wo", "dY"))
+    _, I, rs, _, ws = mosa.mosa_forward(X, Wr, Wq, Wk, Wv, Wo, cfg.k)
+    first = None
+    for _ in range(25):
+        g = mosa.mosa_backward(X, Wr, Wq, Wk, Wv, Wo, I, rs, dY, ws)
+        if first is None:
+            first = g
+        for n in ("dW_r", "dW_q", "dW_k", "dW_v", "dW_o"):
+            assert torch.equal(first[n], g[n]), n
+    ref = oracle.backward(x["X"], *(x[n] for n in ("Wr", "Wq", "Wk", "Wv", "Wo")),
+                          I=I.cpu().numpy(), dY=x["dY"])
+    for n in ("dW_r", "dW_q", "dW_k", "dW_v", "dW_o"):
+        assert_close(n, first[n].cpu().numpy(), ref[n[:2] + n[3:]], cfg.dtype)
