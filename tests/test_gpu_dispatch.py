@@ -105,3 +105,27 @@ def test_non_finite_token_stays_behind_the_mask(cfg, value):
     np.testing.assert_allclose(Yb[1, :at], Y[1, :at], **tol)
     np.testing.assert_allclose(dXb[others], dX[others], **tol)
     np.testing.assert_allclose(dXb[1, at + 1:], dX[1, at + 1:], **tol)
+
+
+# Router on CUDA cores: tiles of 16, 32 and 64 heads and more than one of them, ragged tokens,
+# one chunk of d and several, X at an unaligned address.  A score is one multiply-add
+# chain: at most d roundings of 2^-24 of the sum of |x w|, which sigmoid' = 1/4 at most scales,
+# and the sigmoid's own few.
+@pytest.mark.parametrize("dtype,hp", [("f32", 16), ("bf16", 128)])
+@pytest.mark.parametrize("T,d,H", [(37, 8, 1), (100, 72, 16), (33, 264, 17), (257, 136, 33),
+                                   (64, 520, 65), (95, 104, 130)])
+@pytest.mark.parametrize("unaligned", [False, True])
+def test_router_on_cuda_cores(T, d, H, dtype, hp, unaligned):
+    cfg = W.MosaConfig("router", B=2, T=T, d=d, H=H, hp=hp, k=2, dtype=dtype, seed=107)
+    x = W.make_inputs(cfg, plant=False)
+    X, *w = (to_dev(x[n], dtype) for n in ("X", "Wr", "Wq", "Wk", "Wv", "Wo"))
+    if unaligned:
+        X = shifted(X)
+    _, I, rs, rf, _ = mosa.mosa_forward(X, *w, cfg.k, want_r_full=True)
+    ref = oracle.router(x["X"], x["Wr"])
+    mag = np.einsum("btd,dh->bht", np.abs(x["X"]).astype(np.float64), np.abs(x["Wr"]).astype(np.float64))
+    got = rf.cpu().numpy().astype(np.float64)
+    assert (np.abs(got - ref) <= 2.0 ** -24 * (d * mag / 4 + 8)).all()
+    order = np.argsort(-rf.cpu().numpy(), axis=2, kind="stable")[..., :cfg.k]
+    np.testing.assert_array_equal(I.cpu().numpy(), np.sort(order, axis=2))
+    np.testing.assert_array_equal(rs.cpu().numpy(), np.take_along_axis(rf.cpu().numpy(), np.sort(order, axis=2), axis=2))
