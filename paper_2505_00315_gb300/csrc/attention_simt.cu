@@ -8,8 +8,11 @@
 // (ty, tx) computes RQ x 4 elements of each 16 RQ x 64 score tile and RQ x
 // h'/16 elements of each result, every operand read as float4.  RQ x 4 by 4
 // steps take 16 RQ multiply-adds for RQ + 8 shared-memory wavefronts per
-// thread row, so at RQ = 4 the FMA pipe is the bound (16 against 12 cycles
-// of an SM); smaller tiles trade that for more CTAs.
+// thread row, so at RQ = 4 the FMA pipe has more to do than shared memory (16 against
+// 12 cycles of an SM); smaller tiles trade that for more CTAs.  With eight or sixteen
+// warps on an SM neither is full (ncu, bf16 h' = 128 B4 T1024 H16 k128: forward, RQ = 2, FMA pipe
+// 29% busy, shared memory 64%; backward, RQ = 4, 34% and 47%): the barriers of a tile's loads and
+// the chains between them are what is left.
 //
 // Forward (F4): online softmax; writes A, diag(r^topk) A and the row
 // log-sum-exp.  Backward (B2): P is recomputed from the saved log-sum-exp;

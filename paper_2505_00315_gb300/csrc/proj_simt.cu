@@ -411,7 +411,9 @@ cudaError_t out_t(const Dims &dm, const void *Wo, const Saved &sv, float *Y, cud
 // room for, each of at least three K blocks (the last may find fewer left, none is empty).
 // fp32 at B4 T1000 d768 H12 k125, 48 tiles: 28 -> 15 us on 144 CTAs, its step 225 -> 210.
 // bf16 storage, whose K blocks are only copied, keeps one: at B4 T1024 d1024 H16 h'=128
-// k128, 64 tiles, two splits took 17 -> 13 us here and the step 285.6 -> 286.5.
+// k128, 64 tiles, two splits took 17 -> 13 us here and the step 285.6 -> 286.5.  (At 4 to 48 tiles
+// splits left six steps within 1% and took 203 -> 199 us off one, B2 T1024 d1024 H12 h'=128 k128, and
+// 110.7 -> 105.4 off another, B2 T512 d1024 H16 h'=32 k64: not used yet.)
 int g_split_count(int M, int N, int K, int groups) {
     const int tiles = (M + 127) / 128 * ((N + 127) / 128) * groups, nkb = (K + 63) / 64;
     const int sp = std::max(1, std::min({kGSplits, 152 / tiles, nkb / 3}));

@@ -42,10 +42,10 @@ struct RouterOp {
 // read eight columns of a token at a time; W_r (rows of any alignment) goes through
 // registers, 16 elements per thread, one chunk ahead, into an fp32 tile.  Measured
 // alone: B4 T2048 d1024 H60 193 us with the general 64 x 64 tile product (scalar
-// loads, nothing in flight across its barriers), 42 us now, bound by its issue
-// slots (80% of them used, 60% of those by the multiply-adds; packed
+// loads, nothing in flight across its barriers), 42 us now, most of it its issue
+// slots (67% used over the kernel under ncu, the FMA pipe 46% busy, shared memory 54%; packed
 // fma.rn.f32x2 on X converted in shared memory was slower, 46 us); B1 T1531 d768
-// H12 129 -> 12 us; fp32 B4 T1000 d768 H12 152 -> 14 us.
+// H12 129 -> 12 us; fp32 B4 T1000 d768 H12 152 -> 14 us (a short wave of 125 CTAs: 27% and 16%).
 constexpr int kRouterStages = 4;
 template <int HT>
 struct RouterTile {
