@@ -925,9 +925,9 @@ bool tc_router(const Dims &dm, const void *X, const void *Wr, int wr_cols, float
 // waited until the copies were through (16 us at B16 T1024 d1024 H64 k64, whose
 // step went from 375 to 365 us; B2 T8192 d1024 H32 k256 168.5 -> 164; four
 // units per thread in flight slowed TopK: 371 and 166).  A launch priority above these for
-// TopK and the kernel after it gains nothing more (B16 T1024 d1024 H64 k64 364.2 us with it, 363.3
-// without, B2 T8192 157.3 and 158.4, B4 T4096 d1024 H8 k2048 359.8 and 362.4), and would
-// put them ahead of the caller's other streams.
+// TopK and the kernel after it would gain up to 1.4% more (B16 T1024 d1024 H64 k64 364.2 us with
+// it, 363.3 without; B2 T8192 157.3, 158.4; B4 T4096 d1024 H8 k2048 359.8, 362.4; H128 k128 400, 406),
+// but put them ahead of the caller's other streams.
 constexpr int kSideCta = 256;   // units per CTA
 
 struct F16Copies {
