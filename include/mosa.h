@@ -24,6 +24,10 @@
  *       r_sel     [B,H,k]      fp32, r^topk in the order of I
  *       r_full    [B,H,T]      fp32 router scores of every token
  *       dW_r      [d,H]  dW_q,dW_k,dW_v [H,d,h']  dW_o [H,h',d]   fp32
+ *   - Tensors start at a multiple of their element size.  Of bf16 layers with hp = 64,
+ *     those other than W_r, dW_r, I, r_sel and r_full start at a multiple of 16
+ *     bytes (else MOSA_ERR_INVALID_ARG); where no 16-byte pieces can be moved elsewhere,
+ *     slower kernels run.
  *   - Calls are asynchronous on `stream` (a cudaStream_t, NULL = legacy default
  *     stream).  They return after argument validation and kernel launch.
  *   - mosa_forward, mosa_forward_with_indices, mosa_backward and the hybrid

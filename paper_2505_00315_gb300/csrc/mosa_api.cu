@@ -93,6 +93,15 @@ mosa_status check_workspace(const Dims &dm, void *ws, size_t bytes, Saved *sv) {
     return MOSA_OK;
 }
 
+// The tensor-core path moves every tensor but W_r, dW_r and the per-token scores in 16-byte
+// pieces (TMA, vector loads, stores and reductions): such a call is refused before
+// anything is launched where one (not null) starts elsewhere.
+bool tc_addresses(const Dims &dm, std::initializer_list<const void *> tensors) {
+    uintptr_t u = 0;
+    for (const void *p : tensors) u |= reinterpret_cast<uintptr_t>(p);
+    return (u & 15) == 0 || !use_tc(dm);
+}
+
 mosa_status cuda_status(cudaError_t e) { return e == cudaSuccess ? MOSA_OK : MOSA_ERR_CUDA; }
 
 // Stages of a forward call and of a backward call (timeline slot resets).
@@ -695,6 +704,7 @@ mosa_status mosa_forward(const mosa_shape *shape, const void *X, const void *W_r
     if (st != MOSA_OK) return st;
     if (!X || !W_r || !W_q || !W_k || !W_v || !W_o || !Y || !I || !r_sel)
         return MOSA_ERR_INVALID_ARG;
+    if (!tc_addresses(dm, {X, W_q, W_k, W_v, W_o, Y})) return MOSA_ERR_INVALID_ARG;
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sv.r_full;
@@ -716,6 +726,7 @@ mosa_status mosa_forward_with_indices(const mosa_shape *shape, const void *X, co
     mosa_status st = check_shape(shape, &dm);
     if (st != MOSA_OK) return st;
     if (!X || !W_q || !W_k || !W_v || !W_o || !I || !r_sel || !Y) return MOSA_ERR_INVALID_ARG;
+    if (!tc_addresses(dm, {X, W_q, W_k, W_v, W_o, Y})) return MOSA_ERR_INVALID_ARG;
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
     const int prio = priority_index((cudaStream_t)stream);
@@ -737,6 +748,8 @@ mosa_status mosa_backward(const mosa_shape *shape, const void *X, const void *W_
     if (st != MOSA_OK) return st;
     if (!X || !W_r || !W_q || !W_k || !W_v || !W_o || !I || !r_sel || !dY || !dX || !dW_r ||
         !dW_q || !dW_k || !dW_v || !dW_o)
+        return MOSA_ERR_INVALID_ARG;
+    if (!tc_addresses(dm, {X, W_q, W_k, W_v, W_o, dY, dX, dW_q, dW_k, dW_v, dW_o}))
         return MOSA_ERR_INVALID_ARG;
     Saved sv;
     if ((st = check_workspace(dm, workspace, workspace_bytes, &sv)) != MOSA_OK) return st;
@@ -769,6 +782,9 @@ mosa_status mosa_hybrid_forward(const mosa_hybrid_shape *shape, const void *X, c
     if (!X || !W_r || !W_q || !W_k || !W_v || !W_o || !Y || !I || !r_sel)
         return MOSA_ERR_INVALID_ARG;
     if (h.has_dense && (!D_q || !D_k || !D_v || !D_o)) return MOSA_ERR_INVALID_ARG;
+    if (!tc_addresses(h.sparse, {X, W_q, W_k, W_v, W_o, Y}) ||
+        (h.has_dense && !tc_addresses(h.dense, {D_q, D_k, D_v, D_o})))
+        return MOSA_ERR_INVALID_ARG;
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;
     float *rf = r_full ? r_full : sp.sparse.r_full;
@@ -817,6 +833,9 @@ mosa_status mosa_hybrid_backward(const mosa_hybrid_shape *shape, const void *X, 
         !dW_q || !dW_k || !dW_v || !dW_o)
         return MOSA_ERR_INVALID_ARG;
     if (h.has_dense && (!D_q || !D_k || !D_v || !D_o || !dD_q || !dD_k || !dD_v || !dD_o))
+        return MOSA_ERR_INVALID_ARG;
+    if (!tc_addresses(h.sparse, {X, W_q, W_k, W_v, W_o, dY, dX, dW_q, dW_k, dW_v, dW_o}) ||
+        (h.has_dense && !tc_addresses(h.dense, {D_q, D_k, D_v, D_o, dD_q, dD_k, dD_v, dD_o})))
         return MOSA_ERR_INVALID_ARG;
     HybridSpace sp;
     if ((st = check_hybrid_workspace(h, workspace, workspace_bytes, &sp)) != MOSA_OK) return st;

@@ -129,3 +129,66 @@ def test_router_on_cuda_cores(T, d, H, dtype, hp, unaligned):
     order = np.argsort(-rf.cpu().numpy(), axis=2, kind="stable")[..., :cfg.k]
     np.testing.assert_array_equal(I.cpu().numpy(), np.sort(order, axis=2))
     np.testing.assert_array_equal(rs.cpu().numpy(), np.take_along_axis(rf.cpu().numpy(), np.sort(order, axis=2), axis=2))
+
+
+# bf16 layers with heads of 64 move their tensors in 16-byte pieces only: such a tensor at another
+# address is refused before anything is launched; W_r, dW_r and the scores may lie anywhere
+@pytest.mark.parametrize("hybrid", [False, True])
+@pytest.mark.parametrize("k", [32, 160])
+def test_unaligned_tensors_of_tensor_core_layers_are_refused(k, hybrid):
+    cfg = W.MosaConfig("refused", B=2, T=320, d=72, H=8, hp=64, k=k, dtype="bf16", seed=108)
+    x = W.make_inputs(cfg)
+    t = {n: to_dev(x[s], "bf16") for n, s in
+         {"X": "X", "W_r": "Wr", "W_q": "Wq", "W_k": "Wk", "W_v": "Wv", "W_o": "Wo", "dY": "dY"}.items()}
+    names = ["X", "W_r", "W_q", "W_k", "W_v", "W_o"]
+    kw = {}
+    if hybrid:
+        for n, a in W.make_dense_weights(cfg, 2).items():
+            t["D_" + n[1]] = to_dev(a, "bf16")
+        names += ["D_q", "D_k", "D_v", "D_o"]
+        kw = {"window": 160}
+    forward = mosa.mosa_hybrid_forward if hybrid else mosa.mosa_forward
+    backward = mosa.mosa_hybrid_backward if hybrid else mosa.mosa_backward
+
+    def fresh():
+        return ({"Y": torch.empty(t["X"].shape, device="cuda"),
+                 "I": torch.empty((cfg.B, cfg.H, k), dtype=torch.int32, device="cuda"),
+                 "r_sel": torch.empty((cfg.B, cfg.H, k), device="cuda")},
+                {"d" + n: torch.empty(t[n].shape, device="cuda") for n in names})
+
+    out, grads = fresh()
+    got = forward(*(t[n] for n in names), k, out=out, **kw)
+    ws, I, rs = got[-1], got[1], got[2]
+    ref = {n: g.clone() for n, g in backward(*(t[n] for n in names), I, rs, t["dY"], ws, out=grads, **kw).items()}
+    ref["Y"] = out["Y"].clone()
+    torch.cuda.synchronize()
+
+    anywhere = ("W_r", "dW_r", "I", "r_sel")
+    for n in names + ["Y", "I", "r_sel"]:
+        a, (o, _) = dict(t), fresh()
+        group = o if n in o else a
+        group[n] = shifted(group[n])
+        before = mosa.mosa_kernel_launches()
+        if n in anywhere:
+            y = forward(*(a[m] for m in names), k, workspace=ws, out=o, **kw)[0]
+            torch.testing.assert_close(y, ref["Y"], rtol=1e-4, atol=1e-4)
+            continue
+        with pytest.raises(RuntimeError, match="INVALID_ARG"):
+            forward(*(a[m] for m in names), k, workspace=ws, out=o, **kw)
+        assert mosa.mosa_kernel_launches() == before, n
+    forward(*(t[n] for n in names), k, workspace=ws, out=out, **kw)
+    for n in names + ["dY"] + ["d" + m for m in names]:
+        if n == "W_r":
+            continue
+        a, (_, g) = dict(t), fresh()
+        group = g if n in g else a
+        group[n] = shifted(group[n])
+        before = mosa.mosa_kernel_launches()
+        if n in anywhere:
+            got = backward(*(a[m] for m in names), I, rs, a["dY"], ws, out=g, **kw)
+            torch.testing.assert_close(got[n], ref[n], rtol=1e-3, atol=1e-4)
+            continue
+        with pytest.raises(RuntimeError, match="INVALID_ARG"):
+            backward(*(a[m] for m in names), I, rs, a["dY"], ws, out=g, **kw)
+        assert mosa.mosa_kernel_launches() == before, n
+    assert mosa.mosa_check_status(mosa.make_shape(t["X"], t["W_q"], k), ws) == 0
